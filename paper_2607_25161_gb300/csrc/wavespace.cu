@@ -13,14 +13,16 @@
 // FSD_SPREAD_ATOMIC=1: bead-centric k_spread / k_spread_v4 (warp-wide and
 // 16-byte vector atomic adds into zeroed fields).
 //
-// FFT.  The forward pass turns the six real fields into half spectra
-// [6][n][n][n/2 + 1] (complex, planar per component).  FP32 planes that fit
-// in shared memory run fused x + y kernels (k_fft_xy_fwd / k_fft_xy_inv, one
-// 1024-thread block per (component, z) plane, radix-16 / 9 / 8 register
-// DFTs) and the inverse writes planar velocity fields [6][n^3]; larger
-// grids and FP64 take separate x and y passes (the same radix-16 / 9 / 8
-// plans) and interleaved velocity fields [n^3][8].  k_fft_z_green does the z transforms with the
-// Green's function applied between forward and inverse.
+// FFT.  Sizes that factor into two register DFTs (fft.cuh; every even
+// 2,3,5-smooth size up to 400 but 250 and 384) run as one pass per axis on
+// three complex fields g_p + i g_(p+3), with the Green's function between the
+// forward and inverse z transforms; the inverse leaves planar velocity fields
+// [6][n^3] (FP32) or interleaved ones [n^3][8] (FP64).  On the 32768-bead
+// benchmark (n = 144, FP32) the five passes take 0.165 ms against 0.243 for
+// the fused plane kernels and staged z pass they replaced, 0.62 against 1.31
+// ms at n = 216 and, in FP64, 0.71 against 1.08 ms at n = 96.  Other sizes
+// take the staged plan: half spectra [6][n][n][n/2 + 1] and interleaved
+// velocity fields.
 //   comps 0..2  monopole density g_F = sum_j F_j W(x - x_j)
 //   comps 3..5  dipole density   g_D = sum_j 2 alpha W(x - x_j) D_j (x - x_j),
 //                D = S + A, A y = (1/2) L x y
@@ -31,8 +33,8 @@
 // read-outs: velocity from fM u_hat, rotation / strain from grad (fD u_hat)
 // (k_interp_v4 for FP32 planar fields on grids that are multiples of 4,
 // k_interp for other FP32 planar fields, k_interp_rows for interleaved
-// fields: FP64 and the large FP32 grids).
-#include "fsd_internal.cuh"
+// fields: FP64 and the staged plan's).
+#include "fft.cuh"
 
 #include <algorithm>
 #include <mutex>
@@ -343,56 +345,6 @@ __device__ Cx<T> *fft_lines(Cx<T> *A, Cx<T> *B, int nl, int n, int ls, const Fft
   return in;
 }
 
-// The 144-point transform (radix 16 then 9) on lines of stride kLS144 = 153
-// (= 9 mod 16): the first stage reads the lines in natural order and writes
-// padded order (element i at i + i/16), the second reads padded order and
-// writes natural order back into A.  Every access is a fixed offset from the
-// butterfly's base address (no per-element index arithmetic), and neither
-// stage has shared-memory bank conflicts: in natural order the lanes of a
-// half-warp read 16 consecutive elements of one or two lines, 153 apart; the
-// padding spreads the first stage's stride-16 writes and the second stage's
-// stride-16 reads.  tw2: the second stage's twiddles exp(-2 pi i r j / 144),
-// [r - 1][j], r < 9, j < 16.
-constexpr int kLS144 = 153;
-
-template <typename T>
-__device__ __forceinline__ void fft144_lines(Cx<T> *A, Cx<T> *B, int nl, const Cx<T> *tw2, T sg) {
-  for (int b = threadIdx.x; b < nl * 9; b += blockDim.x) {
-    const int line = b / 9, j = b - line * 9;
-    const Cx<T> *src = A + line * kLS144 + j;
-    Cx<T> v[16];
-#pragma unroll
-    for (int r = 0; r < 16; ++r) v[r] = src[9 * r];
-    dft_small<T, 16>(v, sg);
-    Cx<T> *dst = B + line * kLS144 + 17 * j;
-#pragma unroll
-    for (int r = 0; r < 16; ++r) dst[r] = v[r];
-  }
-  __syncthreads();
-  for (int b = threadIdx.x; b < nl * 16; b += blockDim.x) {
-    const int line = b >> 4, j = b & 15;
-    const Cx<T> *src = B + line * kLS144 + j;
-    Cx<T> v[9];
-    v[0] = src[0];
-#pragma unroll
-    for (int r = 1; r < 9; ++r) {
-      Cx<T> w = tw2[(r - 1) * 16 + j];
-      w.y *= -sg;  // tables hold the forward twiddles
-      v[r] = cmul(src[17 * r], w);
-    }
-    dft_small<T, 9>(v, sg);
-    Cx<T> *dst = A + line * kLS144 + j;
-#pragma unroll
-    for (int r = 0; r < 9; ++r) dst[16 * r] = v[r];
-  }
-  __syncthreads();
-}
-
-// Plans served by fft144_lines: n = 144 as 16 x 9 with lines of stride 153.
-__host__ __device__ __forceinline__ bool is_fft144(const FftPlan &p) {
-  return p.n == 144 && p.nst == 2 && p.st[0].R == 16 && p.st[1].R == 9 && fft_ls(144) == kLS144;
-}
-
 template <typename T>
 __device__ __forceinline__ void load_twiddles(Cx<T> *tw_s, const T *__restrict__ tw, int ntw) {
   for (int t = threadIdx.x; t < ntw; t += blockDim.x) tw_s[t] = {tw[2 * t], tw[2 * t + 1]};
@@ -591,148 +543,6 @@ __global__ void k_fft_y(Cx<T> *spec, FftPlan plan, const T *__restrict__ tw, int
   }
 }
 
-// ------------------------------------------------ fused x + y passes (FP32)
-// One block per (component, z) plane, both transforms in shared memory
-// (FP32 planes up to n = 160 fit next to their ping-pong copy).
-// Forward: rows y = 2r and 2r + 1 of the real plane form the complex line
-// z_r = g_2r + i g_2r+1; after the x DFT the half spectra of the two rows are
-// A_k = (Z_k + conj Z_{n-k})/2 and B_k = (Z_k - conj Z_{n-k})/(2i), k <= n/2.
-// They are transposed into nh = n/2 + 1 lines along y, transformed, and
-// written as spec[comp][z][y][kx].
-template <typename T, bool S144>
-__global__ void __launch_bounds__(1024) k_fft_xy_fwd(const T *__restrict__ grid, Cx<T> *spec,
-                                                    FftPlan plan, const T *__restrict__ tw) {
-  extern __shared__ unsigned char smem_raw[];
-  const int n = plan.n, ls = fft_ls(n), nh = n / 2 + 1, nr = n / 2;
-  // element i of a line: natural order for the 144-point path, padded else
-  auto P = [](int i) { return S144 ? i : fpad(i); };
-  Cx<T> *tw_s = (Cx<T> *)smem_raw;
-  Cx<T> *A = tw_s + plan.ntw;  // nh lines of ls
-  Cx<T> *B = A + nh * ls;
-  load_twiddles(tw_s, tw, plan.ntw);
-  const int64_t cz = blockIdx.x;  // comp * n + z
-  const T *g = grid + cz * n * n;
-  {
-    // eight loads in flight per thread: the plane load is latency-bound
-    constexpr int U = 8;
-    const int total = nr * n;
-    for (int e0 = threadIdx.x; e0 < total; e0 += U * blockDim.x) {
-      T va[U], vb[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int e = e0 + u * blockDim.x;
-        const int r = (int)fdiv((uint32_t)e, plan.fn), x = e - r * n;
-        va[u] = e < total ? g[(2 * r) * n + x] : T(0);
-        vb[u] = e < total ? g[(2 * r + 1) * n + x] : T(0);
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int e = e0 + u * blockDim.x;
-        if (e >= total) continue;
-        const int r = (int)fdiv((uint32_t)e, plan.fn), x = e - r * n;
-        A[r * ls + P(x)] = {va[u], vb[u]};
-      }
-    }
-  }
-  __syncthreads();
-  Cx<T> *Z, *Y;
-  if constexpr (S144) {
-    fft144_lines<T>(A, B, nr, tw_s + plan.st[1].toff, T(-1));
-    Z = A;
-    Y = B;
-  } else {
-    Z = fft_lines<T>(A, B, nr, n, ls, plan, tw_s, T(-1));
-    Y = (Z == A) ? B : A;
-  }
-  for (int e = threadIdx.x; e < nr * nh; e += blockDim.x) {
-    const int r = (int)fdiv((uint32_t)e, plan.fnh), k = e - r * nh;
-    const Cx<T> zk = Z[r * ls + P(k)];
-    const Cx<T> zm = Z[r * ls + P(k == 0 ? 0 : n - k)];
-    Y[k * ls + P(2 * r)] = {T(0.5) * (zk.x + zm.x), T(0.5) * (zk.y - zm.y)};
-    Y[k * ls + P(2 * r + 1)] = {T(0.5) * (zk.y + zm.y), T(-0.5) * (zk.x - zm.x)};
-  }
-  __syncthreads();
-  Cx<T> *R;
-  if constexpr (S144) {
-    fft144_lines<T>(Y, Z, nh, tw_s + plan.st[1].toff, T(-1));
-    R = Y;
-  } else {
-    R = fft_lines<T>(Y, Z, nh, n, ls, plan, tw_s, T(-1));
-  }
-  Cx<T> *out = spec + cz * n * nh;
-  for (int e = threadIdx.x; e < n * nh; e += blockDim.x) {
-    const int y = (int)fdiv((uint32_t)e, plan.fnh), k = e - y * nh;
-    out[e] = R[k * ls + P(y)];
-  }
-}
-
-// Inverse of k_fft_xy_fwd: the y lines are transformed back, rows 2r and
-// 2r + 1 are packed as Z_k = A_k + i B_k (k <= n/2; conj(A_{n-k}) +
-// i conj(B_{n-k}) beyond), and the inverse x DFT gives the two real rows as
-// its real and imaginary parts, written to a planar field [comp][z][y][x].
-template <typename T, bool S144>
-__global__ void __launch_bounds__(1024) k_fft_xy_inv(T *field, const Cx<T> *__restrict__ spec,
-                                                    FftPlan plan, const T *__restrict__ tw) {
-  extern __shared__ unsigned char smem_raw[];
-  const int n = plan.n, ls = fft_ls(n), nh = n / 2 + 1, nr = n / 2;
-  auto P = [](int i) { return S144 ? i : fpad(i); };
-  Cx<T> *tw_s = (Cx<T> *)smem_raw;
-  Cx<T> *A = tw_s + plan.ntw;
-  Cx<T> *B = A + nh * ls;
-  load_twiddles(tw_s, tw, plan.ntw);
-  const int64_t cz = blockIdx.x;
-  const Cx<T> *in = spec + cz * n * nh;
-  {
-    constexpr int U = 8;
-    const int total = n * nh;
-    for (int e0 = threadIdx.x; e0 < total; e0 += U * blockDim.x) {
-      Cx<T> v[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int e = e0 + u * blockDim.x;
-        v[u] = e < total ? in[e] : Cx<T>{T(0), T(0)};
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int e = e0 + u * blockDim.x;
-        if (e >= total) continue;
-        const int y = (int)fdiv((uint32_t)e, plan.fnh), k = e - y * nh;
-        A[k * ls + P(y)] = v[u];
-      }
-    }
-  }
-  __syncthreads();
-  Cx<T> *Y, *Z;
-  if constexpr (S144) {
-    fft144_lines<T>(A, B, nh, tw_s + plan.st[1].toff, T(1));
-    Y = A;
-    Z = B;
-  } else {
-    Y = fft_lines<T>(A, B, nh, n, ls, plan, tw_s, T(1));
-    Z = (Y == A) ? B : A;
-  }
-  for (int e = threadIdx.x; e < nr * n; e += blockDim.x) {
-    const int r = (int)fdiv((uint32_t)e, plan.fn), k = e - r * n;
-    const int kk = k <= n / 2 ? k : n - k;
-    const Cx<T> a = Y[kk * ls + P(2 * r)], b = Y[kk * ls + P(2 * r + 1)];
-    Z[r * ls + P(k)] = k <= n / 2 ? Cx<T>{a.x - b.y, a.y + b.x} : Cx<T>{a.x + b.y, -a.y + b.x};
-  }
-  __syncthreads();
-  Cx<T> *X;
-  if constexpr (S144) {
-    fft144_lines<T>(Z, Y, nr, tw_s + plan.st[1].toff, T(1));
-    X = Z;
-  } else {
-    X = fft_lines<T>(Z, Y, nr, n, ls, plan, tw_s, T(1));
-  }
-  T *o = field + cz * n * n;
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    const int y = (int)fdiv((uint32_t)e, plan.fn), x = e - y * n;
-    const Cx<T> v = X[(y >> 1) * ls + P(x)];
-    o[e] = (y & 1) ? v.y : v.x;
-  }
-}
-
 // ------------------------------------------------------- z pass + Green
 // Lines along z for fixed y, TX = 2^LTX consecutive kx, all six components:
 // forward DFT, Green's function, inverse DFT.
@@ -762,32 +572,17 @@ __device__ __forceinline__ void green_le(const GreenLE &g, double mp, double ms,
   t3 = A * fd * fd;
 }
 
-// z index of the q-th row a z-pass block visits: on the 144-point path the
-// rows of each group of 16 are visited in 4 x 4 transposed order (q = 4a + b
-// -> z = 4b + a), so that the 4 kx columns x 4 rows of a half-warp's
-// shared-memory accesses (lines 153 = 9 mod 16 elements apart) fall in 16
-// distinct banks; the sheared Green's table is stored in the same visiting
-// order.  The map is its own inverse.
-template <bool S144>
-__host__ __device__ __forceinline__ int zorder(int q) {
-  if constexpr (S144)
-    return (q & ~15) | ((q & 3) << 2) | ((q >> 2) & 3);
-  else
-    return q;
-}
-
 // Lees-Edwards Green factors for every half-spectrum point, laid out as the
-// z pass visits them: [ky index][kx][kz in visiting order (zorder)][3].
+// z pass visits them: [kx][kz][ky][3] for the two-factor passes (two != 0),
+// [ky][kx][kz][3] for the staged plan.
 template <typename T>
-__global__ void k_green_le_table(int n, GreenLE le, T *gle, int s144) {
+__global__ void k_green_le_table(int n, GreenLE le, T *gle, int two) {
   const int nh = n / 2 + 1;
   const int64_t total = (int64_t)n * nh * n;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int zq = (int)(e % n);
-    const int zz = s144 ? zorder<true>(zq) : zq;
-    const int kx = (int)((e / n) % nh);
-    const int yy = (int)(e / ((int64_t)n * nh));
+    const int lo = (int)(e % n), mid = (int)((e / n) % (two ? n : nh)), hi = (int)(e / ((int64_t)n * (two ? n : nh)));
+    const int kx = two ? hi : mid, yy = two ? lo : hi, zz = two ? mid : lo;
     const int ky = yy <= n / 2 ? yy : yy - n, kz = zz <= n / 2 ? zz : zz - n;
     const int m = kx * kx + ky * ky + kz * kz;
     double g1 = 0.0, g2 = 0.0, g3 = 0.0;
@@ -802,7 +597,7 @@ __global__ void k_green_le_table(int n, GreenLE le, T *gle, int s144) {
   }
 }
 
-template <typename T, bool S144>
+template <typename T>
 __global__ void k_fft_z_green(Cx<T> *spec, FftPlan plan, const T *__restrict__ tw,
                               const T *__restrict__ green, int LTX, GreenLE le,
                               const T *__restrict__ gle) {
@@ -810,7 +605,6 @@ __global__ void k_fft_z_green(Cx<T> *spec, FftPlan plan, const T *__restrict__ t
   const int n = plan.n, ls = fft_ls(n), nh = n / 2 + 1;
   const int TX = 1 << LTX;
   const int NLn = 6 * TX;
-  auto P = [](int i) { return S144 ? i : fpad(i); };
   Cx<T> *tw_s = (Cx<T> *)smem_raw;
   Cx<T> *A = tw_s + plan.ntw;
   Cx<T> *B = A + NLn * ls;
@@ -830,7 +624,7 @@ __global__ void k_fft_z_green(Cx<T> *spec, FftPlan plan, const T *__restrict__ t
       for (int u = 0; u < U; ++u) {
         const int e = e0 + u * blockDim.x;
         const int t = e & (TX - 1), rest = e >> LTX;
-        const int comp = (int)fdiv((uint32_t)rest, plan.fn), zz = zorder<S144>(rest - comp * n);
+        const int comp = (int)fdiv((uint32_t)rest, plan.fn), zz = rest - comp * n;
         const int kx = kx0 + t;
         v[u] = (e < total && kx < nh) ? g[comp * cstride + zz * zstride + (int64_t)yy * nh + kx]
                                       : Cx<T>{T(0), T(0)};
@@ -840,32 +634,26 @@ __global__ void k_fft_z_green(Cx<T> *spec, FftPlan plan, const T *__restrict__ t
         const int e = e0 + u * blockDim.x;
         if (e >= total) continue;
         const int t = e & (TX - 1), rest = e >> LTX;
-        const int comp = (int)fdiv((uint32_t)rest, plan.fn), zz = zorder<S144>(rest - comp * n);
-        A[(comp * TX + t) * ls + P(zz)] = v[u];
+        const int comp = (int)fdiv((uint32_t)rest, plan.fn), zz = rest - comp * n;
+        A[(comp * TX + t) * ls + fpad(zz)] = v[u];
       }
     }
   }
   __syncthreads();
-  Cx<T> *Z;
-  if constexpr (S144) {
-    fft144_lines<T>(A, B, NLn, tw_s + plan.st[1].toff, T(-1));
-    Z = A;
-  } else {
-    Z = fft_lines<T>(A, B, NLn, n, ls, plan, tw_s, T(-1));
-  }
+  Cx<T> *Z = fft_lines<T>(A, B, NLn, n, ls, plan, tw_s, T(-1));
   // Green's function, one (kx, ky, kz) per thread iteration
   const int ky = yy <= n / 2 ? yy : yy - n;
   const double le_tau = le.dev ? *le.dev * le.invL : le.tau;
   for (int e = threadIdx.x; e < (n << LTX); e += blockDim.x) {
-    const int t = e & (TX - 1), zq = e >> LTX, zz = zorder<S144>(zq);
+    const int t = e & (TX - 1), zz = e >> LTX;
     const int kx = kx0 + t;
     const int kz = zz <= n / 2 ? zz : zz - n;
     const int m = kx * kx + ky * ky + kz * kz;
     Cx<T> gF[3], gD[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      gF[d] = Z[(d * TX + t) * ls + P(zz)];
-      gD[d] = Z[((d + 3) * TX + t) * ls + P(zz)];
+      gF[d] = Z[(d * TX + t) * ls + fpad(zz)];
+      gD[d] = Z[((d + 3) * TX + t) * ls + fpad(zz)];
     }
     Cx<T> oM[3] = {{T(0), T(0)}, {T(0), T(0)}, {T(0), T(0)}};
     Cx<T> oD[3] = {{T(0), T(0)}, {T(0), T(0)}, {T(0), T(0)}};
@@ -888,7 +676,7 @@ __global__ void k_fft_z_green(Cx<T> *spec, FftPlan plan, const T *__restrict__ t
         const double kyp = (double)ky - le_tau * (double)kx;
         const double mp = (double)kx * kx + kyp * kyp + (double)kz * kz;
         // factors of this box offset, tabulated once per offset
-        const T *gq = gle + 3 * (((size_t)yy * nh + kx) * n + zq);
+        const T *gq = gle + 3 * (((size_t)yy * nh + kx) * n + zz);
         t1 = gq[0];
         t2 = gq[1];
         t3 = gq[2];
@@ -915,25 +703,19 @@ __global__ void k_fft_z_green(Cx<T> *spec, FftPlan plan, const T *__restrict__ t
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      Z[(d * TX + t) * ls + P(zz)] = oM[d];
-      Z[((d + 3) * TX + t) * ls + P(zz)] = oD[d];
+      Z[(d * TX + t) * ls + fpad(zz)] = oM[d];
+      Z[((d + 3) * TX + t) * ls + fpad(zz)] = oD[d];
     }
   }
   __syncthreads();
   Cx<T> *O = Z;
   Cx<T> *other = (Z == A) ? B : A;
-  Cx<T> *R;
-  if constexpr (S144) {
-    fft144_lines<T>(O, other, NLn, tw_s + plan.st[1].toff, T(1));
-    R = O;
-  } else {
-    R = fft_lines<T>(O, other, NLn, n, ls, plan, tw_s, T(1));
-  }
+  Cx<T> *R = fft_lines<T>(O, other, NLn, n, ls, plan, tw_s, T(1));
   for (int e = threadIdx.x; e < NLn * n; e += blockDim.x) {
     const int t = e & (TX - 1), rest = e >> LTX;
-    const int comp = (int)fdiv((uint32_t)rest, plan.fn), zz = zorder<S144>(rest - comp * n);
+    const int comp = (int)fdiv((uint32_t)rest, plan.fn), zz = rest - comp * n;
     const int kx = kx0 + t;
-    if (kx < nh) g[comp * cstride + zz * zstride + (int64_t)yy * nh + kx] = R[(comp * TX + t) * ls + P(zz)];
+    if (kx < nh) g[comp * cstride + zz * zstride + (int64_t)yy * nh + kx] = R[(comp * TX + t) * ls + fpad(zz)];
   }
 }
 
@@ -1749,9 +1531,19 @@ void build_wave(Ctx &c) {
   c.op32.gout.alloc(osize);
   c.op64.spec.alloc(ssize);
   c.op32.spec.alloc(ssize);
-  // per-stage twiddle tables of the plan
+  // twiddles exp(-2 pi i j k1 / n), [k1 < R1][j < R2], of the two-factor
+  // passes, or the per-stage tables of the staged plan
   std::vector<double> tw;
-  make_plan(n, &tw, true);
+  if (const FftOps<double> *f = fft_ops<double>(n)) {
+    for (int k1 = 0; k1 < f->R1; ++k1)
+      for (int j = 0; j < f->R2; ++j) {
+        const double ang = -2.0 * kPi * j * k1 / n;
+        tw.push_back(std::cos(ang));
+        tw.push_back(std::sin(ang));
+      }
+  } else {
+    make_plan(n, &tw, true);
+  }
   upload(c.op64.twiddle, tw);
   upload(c.op32.twiddle, tw);
   // Green table by m = kx^2 + ky^2 + kz^2
@@ -1814,8 +1606,7 @@ const float4 *posp<float>(Ctx &c) {
 
 // Raise a kernel's dynamic shared-memory limit once per (kernel, size);
 // thread-safe (contexts may run on several host threads).
-template <typename T>
-static void set_smem(const void *fn, size_t bytes) {
+void raise_smem(const void *fn, size_t bytes) {
   static std::mutex mu;
   static std::vector<std::pair<const void *, size_t>> done;
   std::lock_guard<std::mutex> lock(mu);
@@ -1823,6 +1614,22 @@ static void set_smem(const void *fn, size_t bytes) {
     if (d.first == fn && d.second >= bytes) return;
   FSD_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
   done.push_back({fn, bytes});
+}
+
+template <typename T>
+const FftOps<T> *fft_small_ops(int n);
+template <typename T>
+const FftOps<T> *fft_mid_ops(int n);
+template <typename T>
+const FftOps<T> *fft_large_ops(int n);
+template <typename T>
+const FftOps<T> *fft_huge_ops(int n);
+
+template <typename T>
+const FftOps<T> *fft_ops(int n) {
+  for (auto get : {fft_small_ops<T>, fft_mid_ops<T>, fft_large_ops<T>, fft_huge_ops<T>})
+    if (const FftOps<T> *o = get(n)) return o;
+  return nullptr;
 }
 
 // Largest log2 line count <= want whose two line buffers (lines_per_unit
@@ -1837,55 +1644,46 @@ static int fit_log2_lines(int want, int lines_per_unit, int n, int ntw) {
   throw Invalid{"FFT grid too large for one line per block in shared memory"};
 }
 
-// Inverse y and x transforms of the six fields held in spec (after the z
-// pass), then interpolation: y += h^3 sum W (fields) per bead.
+// Inverse y and x transforms of the fields held in spec (after the z pass),
+// then interpolation: y += h^3 sum W (fields) per bead.
 template <typename T>
-static void wave_tail(Ctx &c, OpData<T> &op, const FftPlan &plan, Cx<T> *spec, double *y) {
+static void wave_tail(Ctx &c, OpData<T> &op, Cx<T> *spec, double *y) {
   const int n = c.n, P = c.P;
   const T h = (T)c.h, alpha = (T)c.alpha;
   const double cn = std::pow(c.alpha / kPi, 1.5);
-  const int nh = n / 2 + 1;
-  const int threads = 256;
-  const int ntw = plan.ntw;
-  const size_t sm_xy = (size_t)(ntw + 2 * nh * fft_ls(n)) * sizeof(Cx<T>);
-  const bool fused = sizeof(T) == 4 && sm_xy <= (size_t)227 * 1024;
-  const int LTXy = fit_log2_lines<T>(sizeof(T) == 8 ? 3 : 4, 1, n, ntw);
-  const int TXy = 1 << LTXy;
-  const size_t smy = (size_t)(ntw + 2 * TXy * fft_ls(n)) * sizeof(Cx<T>);
-  const int blocks_y = 6 * n * ceil_div(nh, TXy);
+  const FftOps<T> *f = fft_ops<T>(n);
   {
-  ProfScope ps(c, PG_FFT);
-  if (fused) {
-    if (is_fft144(plan)) {
-      set_smem<T>((const void *)k_fft_xy_inv<T, true>, sm_xy);
-      k_fft_xy_inv<T, true><<<6 * n, 1024, sm_xy, c.stream>>>(op.gout.p, spec, plan, op.twiddle.p);
+    ProfScope ps(c, PG_FFT);
+    if (f) {
+      f->y_pass(c.stream, (Cplx<T> *)spec, (const Cplx<T> *)op.twiddle.p, true);
+      FSD_LAUNCHED(c);
+      f->x_inv(c.stream, (const Cplx<T> *)spec, op.gout.p, (const Cplx<T> *)op.twiddle.p);
+      FSD_LAUNCHED(c);
+      FSD_CUDA(cudaGetLastError());
     } else {
-      set_smem<T>((const void *)k_fft_xy_inv<T, false>, sm_xy);
-      k_fft_xy_inv<T, false><<<6 * n, 1024, sm_xy, c.stream>>>(op.gout.p, spec, plan, op.twiddle.p);
+      const FftPlan plan = make_plan(n, nullptr, true);
+      const int nh = n / 2 + 1, threads = 256, ntw = plan.ntw;
+      const int LTXy = fit_log2_lines<T>(sizeof(T) == 8 ? 3 : 4, 1, n, ntw);
+      const int TXy = 1 << LTXy;
+      const size_t smy = (size_t)(ntw + 2 * TXy * fft_ls(n)) * sizeof(Cx<T>);
+      // the Brownian wave sample can reach this before any forward pass has
+      // raised the kernel's shared-memory limit
+      raise_smem((const void *)k_fft_y<T>, smy);
+      k_fft_y<T><<<6 * n * ceil_div(nh, TXy), threads, smy, c.stream>>>(spec, plan, op.twiddle.p, LTXy, T(1));
+      FSD_LAUNCHED(c);
+      FSD_CUDA(cudaGetLastError());
+      const int NL = 1 << fit_log2_lines<T>(2, 3, n, ntw);
+      const size_t sm = (size_t)(ntw + 2 * 3 * NL * fft_ls(n)) * sizeof(Cx<T>);
+      raise_smem((const void *)k_fft_x_inv<T>, sm);
+      k_fft_x_inv<T><<<ceil_div((int64_t)n * n, NL), threads, sm, c.stream>>>(op.gout.p, spec, plan,
+                                                                             op.twiddle.p, NL);
+      FSD_LAUNCHED(c);
+      FSD_CUDA(cudaGetLastError());
     }
-    FSD_LAUNCHED(c);
-    FSD_CUDA(cudaGetLastError());
-  } else {
-    // the Brownian wave sample can reach this before any forward pass has
-    // raised the kernel's shared-memory limit
-    set_smem<T>((const void *)k_fft_y<T>, smy);
-    k_fft_y<T><<<blocks_y, threads, smy, c.stream>>>(spec, plan, op.twiddle.p, LTXy, T(1));
-    FSD_LAUNCHED(c);
-    FSD_CUDA(cudaGetLastError());
-    const int NL = 1 << fit_log2_lines<T>(2, 3, n, ntw);
-    size_t sm = (size_t)(ntw + 2 * 3 * NL * fft_ls(n)) * sizeof(Cx<T>);
-    set_smem<T>((const void *)k_fft_x_inv<T>, sm);
-    int blocks = ceil_div((int64_t)n * n, NL);
-    k_fft_x_inv<T><<<blocks, threads, sm, c.stream>>>(op.gout.p, spec, plan, op.twiddle.p, NL);
-    FSD_LAUNCHED(c);
-    FSD_CUDA(cudaGetLastError());
-  }
   }
   ProfScope ps2(c, PG_INTERP);
   const double h3 = c.h * c.h * c.h;
-  const bool planar = sizeof(T) == 4 &&
-                      (size_t)(make_plan(n, nullptr, true).ntw + 2 * (n / 2 + 1) * fft_ls(n)) * sizeof(Cx<T>) <=
-                          (size_t)227 * 1024;
+  const bool planar = sizeof(T) == 4 && f;
   if (planar && n % 4 == 0)
     k_interp_v4<<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p,
                                                          (const float *)op.gout.p, y, n, P,
@@ -1902,7 +1700,6 @@ static void wave_tail(Ctx &c, OpData<T> &op, const FftPlan &plan, Cx<T> *spec, d
   FSD_LAUNCHED(c);
   FSD_CUDA(cudaGetLastError());
 }
-
 
 // Per-tile bead lists of the grid-centric spreading, from the FP32
 // wave-space positions: count, scan, fill, then each list sorted (a fixed
@@ -1982,7 +1779,7 @@ static void refresh_le_table(Ctx &c, OpData<T> &op) {
     le.eta = c.eta;
     le.inv_n3 = 1.0 / ((double)n * n * n);
     k_green_le_table<T><<<4 * c.num_sms, 256, 0, c.stream>>>(
-        n, le, op.green_le.p, is_fft144(make_plan(n, nullptr, true)) ? 1 : 0);
+        n, le, op.green_le.p, fft_ops<T>(n) ? 1 : 0);
   }
   FSD_LAUNCHED(c);
   FSD_CUDA(cudaGetLastError());
@@ -2025,79 +1822,64 @@ void launch_wavespace(Ctx &c, const double *x, double *y) {
   FSD_LAUNCHED(c);
   FSD_CUDA(cudaGetLastError());
   }
-  const FftPlan plan = make_plan(n, nullptr, true);
   Cx<T> *spec = (Cx<T> *)op.spec.p;
+  const bool sheared = c.tilt != 0.0 || tilt_dev_ptr(c);
+  if (sheared) refresh_le_table<T>(c, op);  // once per box offset
   {
   ProfScope ps(c, PG_FFT);
-  const int nh = n / 2 + 1;
-  const int threads = 256;
-  const int ntw = plan.ntw;
-  // FP32 planes that fit in shared memory with their ping-pong copy take the
-  // fused x + y kernels (interpolation then reads planar fields); otherwise
-  // separate x and y passes (interleaved fields).
-  const size_t sm_xy = (size_t)(ntw + 2 * nh * fft_ls(n)) * sizeof(Cx<T>);
-  const bool fused = sizeof(T) == 4 && sm_xy <= (size_t)227 * 1024;
-  const int LTXy = fit_log2_lines<T>(sizeof(T) == 8 ? 3 : 4, 1, n, ntw);
-  const int TXy = 1 << LTXy;
-  const size_t smy = (size_t)(ntw + 2 * TXy * fft_ls(n)) * sizeof(Cx<T>);
-  const int blocks_y = 6 * n * ceil_div(nh, TXy);
-  if (fused) {
-    if (is_fft144(plan)) {
-      set_smem<T>((const void *)k_fft_xy_fwd<T, true>, sm_xy);
-      k_fft_xy_fwd<T, true><<<6 * n, 1024, sm_xy, c.stream>>>(op.grid.p, spec, plan, op.twiddle.p);
-    } else {
-      set_smem<T>((const void *)k_fft_xy_fwd<T, false>, sm_xy);
-      k_fft_xy_fwd<T, false><<<6 * n, 1024, sm_xy, c.stream>>>(op.grid.p, spec, plan, op.twiddle.p);
+  if (const FftOps<T> *f = fft_ops<T>(n)) {
+    const Cplx<T> *tw = (const Cplx<T> *)op.twiddle.p;
+    f->x_fwd(c.stream, op.grid.p, (Cplx<T> *)spec, tw);
+    FSD_LAUNCHED(c);
+    f->y_pass(c.stream, (Cplx<T> *)spec, tw, false);
+    FSD_LAUNCHED(c);
+    ZGreen<T> g;
+    g.green = op.green.p;
+    if (sheared) {
+      g.gle = op.green_le.p;
+      g.tilt_dev = tilt_dev_ptr(c);
+      g.tau = c.tilt / c.L;
+      g.invL = 1.0 / c.L;
     }
+    f->z_green(c.stream, (Cplx<T> *)spec, tw, g);
     FSD_LAUNCHED(c);
     FSD_CUDA(cudaGetLastError());
   } else {
+    const FftPlan plan = make_plan(n, nullptr, true);
+    const int nh = n / 2 + 1, threads = 256, ntw = plan.ntw;
+    const int LTXy = fit_log2_lines<T>(sizeof(T) == 8 ? 3 : 4, 1, n, ntw);
+    const int TXy = 1 << LTXy;
+    const size_t smy = (size_t)(ntw + 2 * TXy * fft_ls(n)) * sizeof(Cx<T>);
     const int NL = 1 << fit_log2_lines<T>(2, 3, n, ntw);
     size_t sm = (size_t)(ntw + 2 * 3 * NL * fft_ls(n)) * sizeof(Cx<T>);
-    set_smem<T>((const void *)k_fft_x_fwd<T>, sm);
-    int blocks = ceil_div((int64_t)n * n, NL);
-    k_fft_x_fwd<T><<<blocks, threads, sm, c.stream>>>(op.grid.p, spec, plan, op.twiddle.p, NL);
+    raise_smem((const void *)k_fft_x_fwd<T>, sm);
+    k_fft_x_fwd<T><<<ceil_div((int64_t)n * n, NL), threads, sm, c.stream>>>(op.grid.p, spec, plan,
+                                                                           op.twiddle.p, NL);
     FSD_LAUNCHED(c);
     FSD_CUDA(cudaGetLastError());
-    set_smem<T>((const void *)k_fft_y<T>, smy);
-    k_fft_y<T><<<blocks_y, threads, smy, c.stream>>>(spec, plan, op.twiddle.p, LTXy, T(-1));
+    raise_smem((const void *)k_fft_y<T>, smy);
+    k_fft_y<T><<<6 * n * ceil_div(nh, TXy), threads, smy, c.stream>>>(spec, plan, op.twiddle.p, LTXy, T(-1));
     FSD_LAUNCHED(c);
     FSD_CUDA(cudaGetLastError());
-  }
-  {
     // four kx columns: 6 x 4 lines keep 4 CTAs per SM (FP32)
     const int LTX = fit_log2_lines<T>(2, 6, n, ntw);
     const int TX = 1 << LTX;
-    size_t sm = (size_t)(ntw + 2 * 6 * TX * fft_ls(n)) * sizeof(Cx<T>);
-    const bool s144 = is_fft144(plan);
-    set_smem<T>(s144 ? (const void *)k_fft_z_green<T, true> : (const void *)k_fft_z_green<T, false>,
-                sm);
-    int blocks = n * ceil_div(nh, TX);
+    sm = (size_t)(ntw + 2 * 6 * TX * fft_ls(n)) * sizeof(Cx<T>);
+    raise_smem((const void *)k_fft_z_green<T>, sm);
     GreenLE le;
-    if (c.tilt != 0.0 || tilt_dev_ptr(c)) {
+    if (sheared) {
       le.on = 1;
       le.tau = c.tilt / c.L;
       le.dev = tilt_dev_ptr(c);
       le.invL = 1.0 / c.L;
-      le.ks2 = (2.0 * kPi / c.L) * (2.0 * kPi / c.L);
-      le.xi = c.xi;
-      le.alpha = c.alpha;
-      le.a = c.a;
-      le.eta = c.eta;
-      le.inv_n3 = 1.0 / ((double)n * n * n);
-      refresh_le_table<T>(c, op);  // once per box offset
     }
-    if (s144)
-      k_fft_z_green<T, true><<<blocks, threads, sm, c.stream>>>(spec, plan, op.twiddle.p,
-                                                                op.green.p, LTX, le, op.green_le.p);
-    else
-      k_fft_z_green<T, false><<<blocks, threads, sm, c.stream>>>(spec, plan, op.twiddle.p,
-                                                                 op.green.p, LTX, le, op.green_le.p);
+    k_fft_z_green<T><<<n * ceil_div(nh, TX), threads, sm, c.stream>>>(spec, plan, op.twiddle.p, op.green.p,
+                                                                      LTX, le, op.green_le.p);
     FSD_LAUNCHED(c);
     FSD_CUDA(cudaGetLastError());
   }
   }
-  wave_tail<T>(c, op, plan, spec, y);
+  wave_tail<T>(c, op, spec, y);
 }
 
 template void launch_wavespace<float>(Ctx &, const double *, double *);
@@ -2107,31 +1889,49 @@ template <typename T>
 void launch_brownian_wave(Ctx &c, const double *field, uint64_t seed, uint64_t step, double *out) {
   OpData<T> &op = opd<T>(c);
   const int n = c.n, nh = n / 2 + 1;
-  const FftPlan plan = make_plan(n, nullptr, true);
   Cx<T> *spec = (Cx<T> *)op.spec.p;
   {
     ProfScope ps(c, PG_FFT);
-    const int LTX = fit_log2_lines<T>(2, 6, n, plan.ntw);
-    const int TX = 1 << LTX;
-    const size_t sm = (size_t)(plan.ntw + 2 * 6 * TX * fft_ls(n)) * sizeof(Cx<T>);
-    set_smem<T>((const void *)k_brown_z<T>, sm);
-    GreenLE le;
-    if (c.tilt != 0.0) {
-      le.tau = c.tilt / c.L;
-      le.ks2 = (2.0 * kPi / c.L) * (2.0 * kPi / c.L);
-      le.xi = c.xi;
-      le.alpha = c.alpha;
-      le.a = c.a;
-      le.eta = c.eta;
-      le.isv = 1.0 / std::sqrt(c.L * c.L * c.L);
+    if (const FftOps<T> *f = fft_ops<T>(n)) {
+      ZBrown<T> b;
+      b.btab = op.btab.p;
+      b.field = field;
+      b.seed = seed;
+      b.step = step;
+      if (c.tilt != 0.0) {
+        b.tau = c.tilt / c.L;
+        b.ks2 = (2.0 * kPi / c.L) * (2.0 * kPi / c.L);
+        b.xi = c.xi;
+        b.alpha = c.alpha;
+        b.a = c.a;
+        b.eta = c.eta;
+        b.isv = 1.0 / std::sqrt(c.L * c.L * c.L);
+      }
+      f->z_brown(c.stream, (Cplx<T> *)spec, (const Cplx<T> *)op.twiddle.p, b);
+    } else {
+      const FftPlan plan = make_plan(n, nullptr, true);
+      const int LTX = fit_log2_lines<T>(2, 6, n, plan.ntw);
+      const int TX = 1 << LTX;
+      const size_t sm = (size_t)(plan.ntw + 2 * 6 * TX * fft_ls(n)) * sizeof(Cx<T>);
+      raise_smem((const void *)k_brown_z<T>, sm);
+      GreenLE le;
+      if (c.tilt != 0.0) {
+        le.tau = c.tilt / c.L;
+        le.ks2 = (2.0 * kPi / c.L) * (2.0 * kPi / c.L);
+        le.xi = c.xi;
+        le.alpha = c.alpha;
+        le.a = c.a;
+        le.eta = c.eta;
+        le.isv = 1.0 / std::sqrt(c.L * c.L * c.L);
+      }
+      k_brown_z<T><<<n * ceil_div(nh, TX), 256, sm, c.stream>>>(spec, plan, op.twiddle.p, op.btab.p, field,
+                                                                 seed, step, LTX, le);
     }
-    k_brown_z<T><<<n * ceil_div(nh, TX), 256, sm, c.stream>>>(spec, plan, op.twiddle.p, op.btab.p,
-                                                               field, seed, step, LTX, le);
     FSD_LAUNCHED(c);
     FSD_CUDA(cudaGetLastError());
   }
   FSD_CUDA(cudaMemsetAsync(out, 0, (size_t)c.nunk * sizeof(double), c.stream));
-  wave_tail<T>(c, op, plan, spec, out);
+  wave_tail<T>(c, op, spec, out);
 }
 template void launch_brownian_wave<float>(Ctx &, const double *, uint64_t, uint64_t, double *);
 template void launch_brownian_wave<double>(Ctx &, const double *, uint64_t, uint64_t, double *);
@@ -2196,54 +1996,17 @@ NaLayout na_layout(int n, int nb) {
   return l;
 }
 
-// FFT plan built without any host container (same stages as make_plan).
-FftPlan na_plan(int n) {
-  FftPlan p{};
-  p.n = n;
-  p.fn = make_fastdiv(n);
-  p.fnh = make_fastdiv(n / 2 + 1);
-  int m = n, k = 0, Ns = 1, off = 0;
-  int rad[kMaxStages];
-  int nr = 0;
-  while (m % 4 == 0) {
-    rad[nr++] = 4;
-    m /= 4;
-  }
-  for (int f : {2, 3, 5})
-    while (m % f == 0) {
-      rad[nr++] = f;
-      m /= f;
-    }
-  for (int i = 0; i < nr; ++i) {
-    FftStage &s = p.st[k++];
-    s.R = rad[i];
-    s.Ns = Ns;
-    s.toff = off;
-    s.nb = make_fastdiv(n / rad[i]);
-    s.ns = make_fastdiv(Ns);
-    off += (rad[i] - 1) * Ns;
-    Ns *= rad[i];
-  }
-  p.nst = k;
-  p.ntw = off;
-  return p;
-}
-
-// Twiddles of the plan and the Green's table (same formulas as build_wave).
-__global__ void k_na_tables(FftPlan plan, float *tw, float *green, int mmax, double L, double xi,
+// Twiddles of the transform and the Green's table (same formulas as build_wave).
+__global__ void k_na_tables(int n, int R2, float *tw, float *green, int mmax, double L, double xi,
                             double alpha, double a, double eta) {
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
   const int stride = gridDim.x * blockDim.x;
-  for (int t = t0; t < plan.ntw; t += stride) {
-    int s = 0;
-    while (s + 1 < plan.nst && plan.st[s + 1].toff <= t) ++s;
-    const int u = t - plan.st[s].toff;
-    const int r = 1 + u / plan.st[s].Ns, kk = u % plan.st[s].Ns;
-    const double ang = -2.0 * kPi * r * kk / ((double)plan.st[s].Ns * plan.st[s].R);
+  for (int t = t0; t < n; t += stride) {
+    const double ang = -2.0 * kPi * (t / R2) * (t % R2) / (double)n;
     tw[2 * t] = (float)cos(ang);
     tw[2 * t + 1] = (float)sin(ang);
   }
-  const double n3 = (double)plan.n * plan.n * plan.n;
+  const double n3 = (double)n * n * n;
   for (int m = t0; m <= mmax; m += stride) {
     if (m == 0) {
       green[0] = green[1] = green[2] = 0.f;
@@ -2348,32 +2111,32 @@ extern "C" fsd_status fsd_apply_wave_noalloc(int64_t n_beads, const double *bead
   const double L = box, h = L / n;
   const double ms = m_shape > 0 ? m_shape : 0.976 * std::sqrt(kPi * P);
   const double alpha = 2.0 * ms * ms / ((P * h) * (P * h));
-  const FftPlan plan = na_plan(n);
+  const FftOps<float> *f = fft_ops<float>(n);  // built for every accepted grid
+  if (!f) return FSD_EINVAL;
   const int hm = n / 2, mmax = 3 * hm * hm;
-  const int nh = n / 2 + 1;
-  const int threads = 256;
-  k_na_tables<<<8, 256, 0, st>>>(plan, tw, green, mmax, L, xi, alpha, a, eta);
+  k_na_tables<<<8, 256, 0, st>>>(n, f->R2, tw, green, mmax, L, xi, alpha, a, eta);
   k_na_stage_in<<<(nb + 127) / 128, 128, 0, st>>>(nb, bead_pos, in, L, pos4, x, y);
   if (cudaMemsetAsync(gridp, 0, (size_t)6 * n * n * n * sizeof(float), st) != cudaSuccess)
     return FSD_ECUDA;
   const double cn = std::pow(alpha / kPi, 1.5);
   k_spread<float><<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, x, gridp, n, P, (float)h, (float)alpha,
                                                (float)cn, TauArg());
-  const int ntw = plan.ntw;
-  k_fft_x_fwd<float><<<(n * n + 3) / 4, threads, (ntw + 2 * 3 * 4 * fft_ls(n)) * sizeof(Cx<float>),
-                       st>>>(gridp, spec, plan, tw, 4);
-  const int blocks_y = 6 * n * ((nh + 15) / 16);
-  const size_t smy = (size_t)(ntw + 2 * 16 * fft_ls(n)) * sizeof(Cx<float>);
-  k_fft_y<float><<<blocks_y, threads, smy, st>>>(spec, plan, tw, 4, -1.f);
-  k_fft_z_green<float, false><<<n * ((nh + 3) / 4), threads,
-                         (ntw + 2 * 6 * 4 * fft_ls(n)) * sizeof(Cx<float>), st>>>(spec, plan, tw,
-                                                                                green, 2, GreenLE(),
-                                                                                nullptr);
-  k_fft_y<float><<<blocks_y, threads, smy, st>>>(spec, plan, tw, 4, 1.f);
-  k_fft_x_inv<float><<<(n * n + 3) / 4, threads, (ntw + 2 * 3 * 4 * fft_ls(n)) * sizeof(Cx<float>),
-                       st>>>(gout, spec, plan, tw, 4);
-  k_interp<float, false><<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha,
-                                               (float)(cn * h * h * h), TauArg());
+  const Cplx<float> *twc = (const Cplx<float> *)tw;
+  Cplx<float> *sp = (Cplx<float> *)spec;
+  ZGreen<float> zg;
+  zg.green = green;
+  f->x_fwd(st, gridp, sp, twc);
+  f->y_pass(st, sp, twc, false);
+  f->z_green(st, sp, twc, zg);
+  f->y_pass(st, sp, twc, true);
+  f->x_inv(st, sp, gout, twc);
+  const float cnh3 = (float)(cn * h * h * h);
+  if (n % 4 == 0)
+    k_interp_v4<<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3, TauArg(),
+                                              make_fastdiv((P + 7) / 4), make_fastdiv(P));
+  else
+    k_interp<float, true><<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3,
+                                                       TauArg());
   k_na_stage_out<<<(nb + 127) / 128, 128, 0, st>>>(nb, y, out);
   if (cudaGetLastError() != cudaSuccess) return FSD_ECUDA;
   return FSD_OK;
