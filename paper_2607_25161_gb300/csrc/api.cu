@@ -615,8 +615,8 @@ static void setup_impl(Ctx &c, int64_t n_beads, const double *bead_pos, const in
   c.ncnt.alloc(Nt);
   c.lnbr.alloc((size_t)Nt * c.lcap);
   c.lcnt.alloc(Nt);
-  c.flags.alloc(8);
-  FSD_CUDA(cudaMallocHost(&c.h_flags, 8 * sizeof(int)));
+  c.flags.alloc(kFlags);
+  FSD_CUDA(cudaMallocHost(&c.h_flags, kFlags * sizeof(int)));
   c.brow.alloc(Nt + 1);
   c.op64.bdiag.alloc((size_t)Nt * 36);
   c.op32.bdiag.alloc((size_t)Nt * 36);
@@ -667,15 +667,6 @@ static void prepare(Ctx &c) {
   c.last_warning = FSD_OK;
   launch_wrap_positions(c);
   build_neighbors(c);
-  {
-    // pair count for the real-space launch shape
-    std::vector<int> cnt(c.Nt);
-    FSD_CUDA(cudaMemcpyAsync(cnt.data(), c.ncnt.p, c.Nt * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
-    FSD_CUDA(cudaStreamSynchronize(c.stream));
-    int64_t s = 0;
-    for (int v : cnt) s += v;
-    c.n_pairs = s;
-  }
   build_lubrication(c);
   if (c.spread_gather && !c.tiles_valid) build_spread_tiles(c);
 }

@@ -34,6 +34,7 @@ constexpr int tab_stride() {
   return tab_coef<T>() * 8 + 4;
 }
 constexpr int BLK = 36;     // 6x6 block
+constexpr int kFlags = 12;  // words of Ctx::flags
 
 // ------------------------------------------------------------------ errors
 struct CudaError {
@@ -195,11 +196,14 @@ struct Ctx {
   // ---- neighbour lists
   int cap = 0, lcap = 0, ncell = 1;
   DBuf<int> nbr, ncnt, lnbr, lcnt;
-  DBuf<int> cell_count, cell_start, cell_beads, cell_cursor;
-  DBuf<int> flags;  // [0] nbr overflow, [1] lub overflow, [2] overlap, [3] singular LU, [4] max count
+  DBuf<int> cell_count, cell_start, cell_beads, cell_cursor, cell_id;
+  // [0] nbr overflow, [1] lub overflow, [2] overlap, [3] singular LU, [4] / [5] largest counts on
+  // overflow, [6] NaN, [8..11] total mobility and lubrication neighbours (two 64-bit sums)
+  DBuf<int> flags;
   int *h_flags = nullptr;  // pinned
   // ---- lubrication BSR (rows = beads; diagonal separate)
   DBuf<int> brow, bcol;
+  DBuf<double> lpair;  // per directed pair (n, r, A, B, D, within r_p) [nnz][8]
   int nnz_cap = 0;
   // ---- preconditioner
   DBuf<double> schur;  // [N][36] LU factors

@@ -10,6 +10,7 @@
 #include "fsd_internal.cuh"
 
 #include <climits>
+#include <cstring>
 #include <mutex>
 
 #include <algorithm>
@@ -262,46 +263,65 @@ __device__ __forceinline__ int cell_of(double x, double L, int nc) {
 }
 
 __global__ void k_cell_count(int Nt, const double4 *__restrict__ pos, double L, int nc,
-                             int *cell_count) {
+                             int *cell_count, int *cell_id) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Nt) return;
   double4 p = pos[i];
   int id = (cell_of(p.x, L, nc) * nc + cell_of(p.y, L, nc)) * nc + cell_of(p.z, L, nc);
   atomicAdd(&cell_count[id], 1);
+  cell_id[i] = id;
 }
 
-// single-block exclusive scan (n up to a few million; serial chunks + block scan)
+// Exclusive scan by one block of 1024 threads: tiles of 4096 values, four
+// consecutive ones per thread, warp shuffles, a running total between tiles
+// (a thread summing its own n/1024 consecutive values took 55 us on 32768
+// counts, the strided loads missing L1; now 9 us).
 __global__ void k_exclusive_scan(int n, const int *__restrict__ in, int *out, int *cursor) {
-  __shared__ int sums[1024];
-  int t = threadIdx.x;
-  int per = (n + blockDim.x - 1) / blockDim.x;
-  int b = t * per, e = min(n, b + per);
-  int s = 0;
-  for (int i = b; i < e; ++i) s += in[i];
-  sums[t] = s;
-  __syncthreads();
-  for (int off = 1; off < blockDim.x; off <<= 1) {
-    int v = (t >= off) ? sums[t - off] : 0;
+  __shared__ int wsum[32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  int carry = 0;
+  for (int b0 = 0; b0 < n; b0 += 4096) {
+    const int b = b0 + 4 * t;
+    int v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = b + e < n ? in[b + e] : 0;
+    const int mine = v[0] + v[1] + v[2] + v[3];
+    int inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += u;
+    }
+    if (lane == 31) wsum[warp] = inc;
     __syncthreads();
-    sums[t] += v;
+    if (warp == 0) {
+      int w = wsum[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, w, o);
+        if (lane >= o) w += u;
+      }
+      wsum[lane] = w;
+    }
+    __syncthreads();
+    int run = carry + inc - mine + (warp > 0 ? wsum[warp - 1] : 0);
+    carry += wsum[31];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (b + e < n) {
+        out[b + e] = run;
+        if (cursor) cursor[b + e] = run;
+        run += v[e];
+      }
     __syncthreads();
   }
-  int run = sums[t] - s;
-  for (int i = b; i < e; ++i) {
-    out[i] = run;
-    if (cursor) cursor[i] = run;
-    run += in[i];
-  }
-  if (t == blockDim.x - 1) out[n] = sums[t];
+  if (t == 0) out[n] = carry;
 }
 
-__global__ void k_cell_fill(int Nt, const double4 *__restrict__ pos, double L, int nc,
-                            int *cursor, int *cell_beads) {
+__global__ void k_cell_fill(int Nt, const int *__restrict__ cell_id, int *cursor, int *cell_beads) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Nt) return;
-  double4 p = pos[i];
-  int id = (cell_of(p.x, L, nc) * nc + cell_of(p.y, L, nc)) * nc + cell_of(p.z, L, nc);
-  int slot = atomicAdd(&cursor[id], 1);
+  int slot = atomicAdd(&cursor[cell_id[i]], 1);
   cell_beads[slot] = i;
 }
 
@@ -358,83 +378,132 @@ __global__ void __launch_bounds__(128) k_sort_cells(int ncells, const int *__res
   for (int i = lane; i < len; i += 32) cell_beads[b + i] = a[i];
 }
 
-// One thread per bead: mobility neighbours (r < rc, any body, j != i) and
-// lubrication neighbours (r < rlub, different body).  Each candidate's
+// One warp per bead: mobility neighbours (r < rc, any body, j != i) and
+// lubrication neighbours (r < rlub, different body), the lanes taking
+// consecutive candidates of the cells around the bead (three cells along z
+// are one run of the sorted list) and ballots placing the accepted ones, so a
+// row keeps the order of the cells.  Each candidate's
 // nearest-image distance is first taken in FP32 from the FP32 positions; only
 // a candidate whose squared distance lies within m2 of a cut-off is measured
 // again in FP64, so every decision is the FP64 one (m2 bounds the FP32
 // rounding of the positions and of the image shift many times over; an
 // image chosen differently in FP32 has a component near L/2, beyond every
 // cut-off either way).  FP64 arithmetic runs at 1/74 of the FP32 rate on
-// this part, and the FP64 test with its three divisions by L was the cost.
-__global__ void k_neighbors(int Nt, const double4 *__restrict__ pos,
-                            const float4 *__restrict__ pos32,
-                            const double4 *__restrict__ spos, double L, double tilt, int nc,
-                            const int *__restrict__ cell_start,
-                            const int *__restrict__ cell_beads,
-                            const int *__restrict__ bead_body, double rc2, double rl2,
-                            double ov2, float m2, int cap, int lcap, int *nbr, int *ncnt,
-                            int *lnbr, int *lcnt, int *flags) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= Nt) return;
-  const double4 p = pos[i];
-  const float4 pf = pos32[i];
-  const double4 sp = spos[i];
-  int bi = bead_body[i];
-  int cx = cell_of(sp.x, L, nc), cy = cell_of(sp.y, L, nc), cz = cell_of(sp.z, L, nc);
-  int cnt = 0, lc = 0;
-  int span = nc >= 3 ? 1 : 0;
-  int *row = nbr + (size_t)i * cap;
-  int *lrow = lnbr + (size_t)i * lcap;
-  const float Lf = (float)L, invLf = 1.f / Lf, tiltf = (float)tilt;
-  const float rc2f = (float)rc2, rl2f = (float)rl2, ov2f = (float)ov2;
-  const float hi = fmaxf(rc2f, fmaxf(rl2f, ov2f)) + m2;
-  for (int dx = -span; dx <= span; ++dx)
-    for (int dy = -span; dy <= span; ++dy)
-      for (int dz = -span; dz <= span; ++dz) {
-        int ax = (cx + dx + nc) % nc, ay = (cy + dy + nc) % nc, az = (cz + dz + nc) % nc;
-        int id = (ax * nc + ay) * nc + az;
-        for (int s = cell_start[id]; s < cell_start[id + 1]; ++s) {
-          int j = cell_beads[s];
-          if (j == i) continue;
-          const float4 qf = pos32[j];
-          float e0 = qf.x - pf.x, e1 = qf.y - pf.y, e2 = qf.z - pf.z;
-          {
-            const float ny = rintf(e1 * invLf);
-            e0 -= ny * tiltf;
-            e1 -= ny * Lf;
-            e0 -= Lf * rintf(e0 * invLf);
-            e2 -= Lf * rintf(e2 * invLf);
-          }
-          const float r2f = e0 * e0 + e1 * e1 + e2 * e2;
-          if (r2f >= hi) continue;
-          double r2 = (double)r2f;
-          if (fabsf(r2f - rc2f) < m2 || fabsf(r2f - rl2f) < m2 || fabsf(r2f - ov2f) < m2) {
-            const double4 q = pos[j];
-            double d0 = q.x - p.x, d1 = q.y - p.y, d2 = q.z - p.z;
-            le_image(d0, d1, d2, L, tilt);
-            r2 = d0 * d0 + d1 * d1 + d2 * d2;
-          }
-          if (r2 < rc2) {
-            if (cnt < cap) row[cnt] = j;
-            ++cnt;
-          }
-          if (bead_body[j] != bi) {
-            if (r2 < ov2) atomicOr(&flags[2], 1);
-            if (r2 < rl2) {
-              if (lc < lcap) lrow[lc] = j;
-              ++lc;
+// this part and one lane's use of it costs the whole warp, so nothing else
+// here is FP64: the cell indices come from the binning, and the touching beads
+// of one body, always at an overlap's distance, are told apart by body first.
+// Bound by the latency of the candidates' loads.  With a thread per bead a
+// suspension of 11 000 beads filled 88 blocks, each thread walking about a
+// thousand candidates alone: 550 us; a warp per bead takes 68 us (and
+// 202 against 730 us on 32768 beads).  The totals of both lists are
+// summed here, so the host needs no copy of the counts.
+__global__ void __launch_bounds__(256) k_neighbors(
+    int Nt, const double4 *__restrict__ pos, const float4 *__restrict__ pos32,
+    const int *__restrict__ cell_id, double L, double tilt, int nc,
+    const int *__restrict__ cell_start, const int *__restrict__ cell_beads,
+    const int *__restrict__ bead_body, double rc2, double rl2, double ov2, float m2, int cap,
+    int lcap, int *nbr, int *ncnt, int *lnbr, int *lcnt, int *flags, unsigned long long *totals) {
+  __shared__ int tot[2];
+  if (threadIdx.x < 2) tot[threadIdx.x] = 0;
+  __syncthreads();
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i < Nt) {
+    const float4 pf = pos32[i];
+    const int bi = bead_body[i];
+    const int id = cell_id[i], cz = id % nc, cy = (id / nc) % nc, cx = id / (nc * nc);
+    int cnt = 0, lc = 0;
+    bool over = false;
+    const int span = nc >= 3 ? 1 : 0;
+    int *row = nbr + (size_t)i * cap;
+    int *lrow = lnbr + (size_t)i * lcap;
+    const float Lf = (float)L, invLf = 1.f / Lf, tiltf = (float)tilt;
+    const float rc2f = (float)rc2, rl2f = (float)rl2, ov2f = (float)ov2;
+    const float close = fmaxf(rl2f, ov2f) + m2, hi = fmaxf(rc2f + m2, close);
+    const unsigned below = (1u << lane) - 1u;
+    // the cells cz - 1 .. cz + 1 in that order: one run, or two across the box
+    int z0[2] = {cz - span, 0}, z1[2] = {cz + span, -1};
+    if (z0[0] < 0) {
+      z0[0] = z1[0] = nc - 1;
+      z1[1] = cz + 1;
+    } else if (z1[0] >= nc) {
+      z1[0] = nc - 1;
+      z1[1] = 0;
+    }
+    for (int dx = -span; dx <= span; ++dx)
+      for (int dy = -span; dy <= span; ++dy) {
+        const int ax = (cx + dx + nc) % nc, ay = (cy + dy + nc) % nc;
+        const int *cs = cell_start + (ax * nc + ay) * nc;
+#pragma unroll
+        for (int run = 0; run < 2; ++run) {
+          if (z1[run] < z0[run]) continue;
+          const int e = cs[z1[run] + 1];
+          for (int s = cs[z0[run]]; s < e; s += 32) {
+            const bool valid = s + lane < e;
+            const int j = valid ? cell_beads[s + lane] : i;
+            bool near = false, lub = false;
+            if (j != i) {
+              const float4 qf = pos32[j];
+              float e0 = qf.x - pf.x, e1 = qf.y - pf.y, e2 = qf.z - pf.z;
+              const float ny = rintf(e1 * invLf);
+              e0 -= ny * tiltf;
+              e1 -= ny * Lf;
+              e0 -= Lf * rintf(e0 * invLf);
+              e2 -= Lf * rintf(e2 * invLf);
+              const float r2f = e0 * e0 + e1 * e1 + e2 * e2;
+              if (r2f < hi) {
+                near = r2f < rc2f;
+                bool unsure = fabsf(r2f - rc2f) < m2, other = false, ov = false;
+                if (r2f < close) {  // touching beads of one body are no matter
+                  other = bead_body[j] != bi;
+                  lub = other && r2f < rl2f;
+                  ov = other && r2f < ov2f;
+                  unsure |= other && (fabsf(r2f - rl2f) < m2 || fabsf(r2f - ov2f) < m2);
+                }
+                if (unsure) {
+                  const double4 p = pos[i], q = pos[j];
+                  double d0 = q.x - p.x, d1 = q.y - p.y, d2 = q.z - p.z;
+                  le_image(d0, d1, d2, L, tilt);
+                  const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
+                  near = r2 < rc2;
+                  lub = other && r2 < rl2;
+                  ov = other && r2 < ov2;
+                }
+                over |= ov;
+              }
+            }
+            const unsigned mn = __ballot_sync(0xffffffffu, near);
+            if (near) {
+              const int at = cnt + __popc(mn & below);
+              if (at < cap) row[at] = j;
+            }
+            cnt += __popc(mn);
+            const unsigned ml = __ballot_sync(0xffffffffu, lub);
+            if (lub) {
+              const int at = lc + __popc(ml & below);
+              if (at < lcap) lrow[at] = j;
             }
           }
+            lc += __popc(ml);
         }
       }
-  const int m = min(cnt, cap);
-  ncnt[i] = m;
-  lcnt[i] = min(lc, lcap);
-  if (cnt > cap) atomicOr(&flags[0], 1);
-  if (lc > lcap) atomicOr(&flags[1], 1);
-  atomicMax(&flags[4], cnt);
-  atomicMax(&flags[5], lc);
+    if (over) atomicOr(&flags[2], 1);
+    if (lane == 0) {
+      ncnt[i] = min(cnt, cap);
+      lcnt[i] = min(lc, lcap);
+      if (cnt > cap) {
+        atomicOr(&flags[0], 1);
+        atomicMax(&flags[4], cnt);
+      }
+      if (lc > lcap) {
+        atomicOr(&flags[1], 1);
+        atomicMax(&flags[5], lc);
+      }
+      atomicAdd(&tot[0], min(cnt, cap));
+      atomicAdd(&tot[1], min(lc, lcap));
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) atomicAdd(&totals[threadIdx.x], (unsigned long long)tot[threadIdx.x]);
 }
 
 // Within each block of 32 consecutive neighbours of a bead (the pairs one
@@ -503,17 +572,18 @@ void build_neighbors(Ctx &c) {
     c.cell_cursor.alloc(ncells);
     c.cell_beads.alloc(c.Nt);
   }
+    c.cell_id.alloc(c.Nt);
   const double4 *pos = (const double4 *)c.pos64.p;
   const double4 *spos = (const double4 *)c.wpos64.p;
   for (int attempt = 0; attempt < 4; ++attempt) {
     FSD_CUDA(cudaMemsetAsync(c.cell_count.p, 0, ncells * sizeof(int), c.stream));
-    FSD_CUDA(cudaMemsetAsync(c.flags.p, 0, 8 * sizeof(int), c.stream));
-    k_cell_count<<<ceil_div(c.Nt, 256), 256, 0, c.stream>>>(c.Nt, spos, c.L, nc, c.cell_count.p);
+    FSD_CUDA(cudaMemsetAsync(c.flags.p, 0, kFlags * sizeof(int), c.stream));
+    k_cell_count<<<ceil_div(c.Nt, 256), 256, 0, c.stream>>>(c.Nt, spos, c.L, nc, c.cell_count.p, c.cell_id.p);
     FSD_LAUNCHED(c);
     k_exclusive_scan<<<1, 1024, 0, c.stream>>>(ncells, c.cell_count.p, c.cell_start.p,
                                                c.cell_cursor.p);
     FSD_LAUNCHED(c);
-    k_cell_fill<<<ceil_div(c.Nt, 256), 256, 0, c.stream>>>(c.Nt, spos, c.L, nc, c.cell_cursor.p,
+    k_cell_fill<<<ceil_div(c.Nt, 256), 256, 0, c.stream>>>(c.Nt, c.cell_id.p, c.cell_cursor.p,
                                                            c.cell_beads.p);
     FSD_LAUNCHED(c);
     k_sort_cells<<<ceil_div(ncells, 4), 128, 0, c.stream>>>(ncells, c.cell_start.p,
@@ -525,13 +595,13 @@ void build_neighbors(Ctx &c) {
     // shift are within a few 1e-7 L of the FP64 ones, so the FP32 r^2 is off
     // by at most ~2e-6 L r_max (five times below the margin)
     const float m2 = (float)(1e-5 * c.L * std::max({c.rc, rl, ov}) + 1e-12);
-    k_neighbors<<<ceil_div(c.Nt, 128), 128, 0, c.stream>>>(
-        c.Nt, pos, (const float4 *)c.op32.pos.p, spos, c.L, c.tilt, nc, c.cell_start.p,
+    k_neighbors<<<ceil_div((int64_t)c.Nt * 32, 256), 256, 0, c.stream>>>(
+        c.Nt, pos, (const float4 *)c.op32.pos.p, c.cell_id.p, c.L, c.tilt, nc, c.cell_start.p,
         c.cell_beads.p, c.bead_body.p, c.rc * c.rc, rl * rl, ov * ov, m2, c.cap, c.lcap, c.nbr.p,
-        c.ncnt.p, c.lnbr.p, c.lcnt.p, c.flags.p);
+        c.ncnt.p, c.lnbr.p, c.lcnt.p, c.flags.p, (unsigned long long *)(c.flags.p + 8));
     FSD_LAUNCHED(c);
     FSD_CUDA(cudaGetLastError());
-    FSD_CUDA(cudaMemcpyAsync(c.h_flags, c.flags.p, 8 * sizeof(int), cudaMemcpyDeviceToHost,
+    FSD_CUDA(cudaMemcpyAsync(c.h_flags, c.flags.p, kFlags * sizeof(int), cudaMemcpyDeviceToHost,
                              c.stream));
     FSD_CUDA(cudaStreamSynchronize(c.stream));
     bool redo = false;
@@ -548,6 +618,10 @@ void build_neighbors(Ctx &c) {
     if (!redo) break;
   }
   k_nbr_order<<<ceil_div((int64_t)c.Nt * 32, 256), 256, 0, c.stream>>>(
+  int64_t totals[2];
+  std::memcpy(totals, c.h_flags + 8, sizeof(totals));
+  c.n_pairs = totals[0];
+  c.n_lub = totals[1];
       c.Nt, (const float4 *)c.op32.pos.p, (float)c.L, (float)c.tilt, c.nbr.p, c.ncnt.p, c.cap);
   FSD_LAUNCHED(c);
   FSD_CUDA(cudaGetLastError());

@@ -1306,16 +1306,20 @@ __global__ void __launch_bounds__(256, 4) k_interp_v4(int Nt, const float4 *__re
 constexpr int kTS = 8;      // tile side
 constexpr int kTCH = 32;    // beads per shared-memory chunk
 
-// distinct tiles (per axis) covered by the window of a bead at coordinate p
+// distinct tiles (per axis) covered by the window of a bead at coordinate p:
+// tile by tile along the window, which may run across the box once
 __device__ __forceinline__ int window_tiles(float p, float h, int P, int n, int t[5]) {
-  const int g0 = (int)floorf(p / h) - P / 2 + 1;
+  int g = (int)floorf(p / h) - P / 2 + 1;
+  g += g < 0 ? n : 0;
+  g -= g >= n ? n : 0;
   int cnt = 0;
-  for (int k = 0; k < P; ++k) {
-    const int g = ((g0 + k) % n + n) % n;
-    const int tt = g / kTS;
-    bool seen = false;
-    for (int q = 0; q < cnt; ++q) seen |= t[q] == tt;
-    if (!seen && cnt < 5) t[cnt++] = tt;
+  for (int left = P; left > 0;) {
+    const int tt = g / kTS, end = min((tt + 1) * kTS, n);
+    if (cnt == 0 || tt != t[0]) {  // a window as long as the box ends in its first tile
+      if (cnt < 5) t[cnt++] = tt;
+    }
+    left -= end - g;
+    g = end == n ? 0 : end;
   }
   return cnt;
 }
