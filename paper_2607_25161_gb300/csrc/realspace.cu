@@ -149,6 +149,7 @@ static std::vector<double> fit_table(const WaveQuad &q, int nint, double ht, int
         tab[(size_t)iv * stride + (size_t)p * 8 + f] = s;
       }
     }
+    tab[(size_t)iv * stride + 7] = 2.0 * iv + 1.0;  // the pad slot of power 0
   }
   return tab;
 }
@@ -268,8 +269,8 @@ __global__ void k_cell_count(int Nt, const double4 *__restrict__ pos, double L, 
   if (i >= Nt) return;
   double4 p = pos[i];
   int id = (cell_of(p.x, L, nc) * nc + cell_of(p.y, L, nc)) * nc + cell_of(p.z, L, nc);
-  atomicAdd(&cell_count[id], 1);
   cell_id[i] = id;
+  atomicAdd(&cell_count[id], 1);
 }
 
 // Exclusive scan by one block of 1024 threads: tiles of 4096 values, four
@@ -482,8 +483,8 @@ __global__ void __launch_bounds__(256) k_neighbors(
               const int at = lc + __popc(ml & below);
               if (at < lcap) lrow[at] = j;
             }
-          }
             lc += __popc(ml);
+          }
         }
       }
     if (over) atomicOr(&flags[2], 1);
@@ -571,8 +572,8 @@ void build_neighbors(Ctx &c) {
     c.cell_start.alloc(ncells + 1);
     c.cell_cursor.alloc(ncells);
     c.cell_beads.alloc(c.Nt);
-  }
     c.cell_id.alloc(c.Nt);
+  }
   const double4 *pos = (const double4 *)c.pos64.p;
   const double4 *spos = (const double4 *)c.wpos64.p;
   for (int attempt = 0; attempt < 4; ++attempt) {
@@ -617,11 +618,11 @@ void build_neighbors(Ctx &c) {
     }
     if (!redo) break;
   }
-  k_nbr_order<<<ceil_div((int64_t)c.Nt * 32, 256), 256, 0, c.stream>>>(
   int64_t totals[2];
   std::memcpy(totals, c.h_flags + 8, sizeof(totals));
   c.n_pairs = totals[0];
   c.n_lub = totals[1];
+  k_nbr_order<<<ceil_div((int64_t)c.Nt * 32, 256), 256, 0, c.stream>>>(
       c.Nt, (const float4 *)c.op32.pos.p, (float)c.L, (float)c.tilt, c.nbr.p, c.ncnt.p, c.cap);
   FSD_LAUNCHED(c);
   FSD_CUDA(cudaGetLastError());
