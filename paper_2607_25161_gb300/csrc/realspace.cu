@@ -720,20 +720,41 @@ __device__ __forceinline__ void free_phi(const T inv, const T a2, const T c8, T 
   ph[6] = c8 * (T(-15) * i7 + T(42) * a2 * i9);
 }
 
-// Wave-part radial functions from the Chebyshev-fitted table (monomials in
-// t in [-1, 1] per interval), all seven functions per Horner step.
+// 1/r and r from r^2: a reciprocal square root estimate refined by one step of
+// Halley's iteration y (1 + e/2 + 3 e^2/8), e = 1 - r^2 y^2, of cubic order: a
+// single-precision estimate reaches FP64 rounding (e^3 ~ 1e-20), and FP32's
+// own estimate FP32 rounding.  One FP64 pipe pass of eight operations instead
+// of a square root and a division (about twenty-five).
 template <typename T>
-__device__ __forceinline__ void wave_table(const T *tab, int nint, T inv_h, T r, T *w);
+__device__ __forceinline__ T inv_sqrt(T r2);
 template <>
-__device__ __forceinline__ void wave_table<float>(const float *tab, int nint, float inv_h, float r,
-                                                  float *w) {
-  const float s = r * inv_h;
-  int iv = (int)s;
+__device__ __forceinline__ float inv_sqrt<float>(float r2) {
+  const float y = rsqrtf(r2), e = fmaf(-r2 * y, y, 1.f);
+  return fmaf(y * e, fmaf(0.375f, e, 0.5f), y);
+}
+template <>
+__device__ __forceinline__ double inv_sqrt<double>(double r2) {
+  const double y = (double)rsqrtf((float)r2), e = fma(-r2 * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// Wave-part radial functions from the Chebyshev-fitted table (monomials in
+// t in [-1, 1] per interval), all seven functions per Horner step.  The pad
+// slot of power 0 holds 2 iv + 1, so that t = 2 r / h - (2 iv + 1) is one
+// operation; the interval itself is found in FP32 in either precision (at an
+// interval's edge t may then pass 1 by an FP32 rounding, where the neighbouring
+// polynomials agree to their fit error).
+template <typename T>
+__device__ __forceinline__ void wave_table(const T *tab, int nint, T two_inv_h, float rf, T r, T *w);
+template <>
+__device__ __forceinline__ void wave_table<float>(const float *tab, int nint, float two_inv_h, float rf,
+                                                  float r, float *w) {
+  int iv = (int)(0.5f * two_inv_h * rf);
   iv = iv < 0 ? 0 : (iv >= nint ? nint - 1 : iv);
-  const float t = 2.f * (s - (float)iv) - 1.f;
   constexpr int NC = tab_coef<float>();
   const float4 *c = (const float4 *)(tab + (size_t)iv * tab_stride<float>());
   float4 lo = c[2 * (NC - 1)], hi = c[2 * (NC - 1) + 1];
+  const float t = fmaf(r, two_inv_h, -(float)(2 * iv + 1));
   float v0 = lo.x, v1 = lo.y, v2 = lo.z, v3 = lo.w, v4 = hi.x, v5 = hi.y, v6 = hi.z;
 #pragma unroll
   for (int p = NC - 2; p >= 0; --p) {
@@ -745,14 +766,13 @@ __device__ __forceinline__ void wave_table<float>(const float *tab, int nint, fl
   w[0] = v0; w[1] = v1; w[2] = v2; w[3] = v3; w[4] = v4; w[5] = v5; w[6] = v6;
 }
 template <>
-__device__ __forceinline__ void wave_table<double>(const double *tab, int nint, double inv_h,
+__device__ __forceinline__ void wave_table<double>(const double *tab, int nint, double two_inv_h, float rf,
                                                    double r, double *w) {
-  const double s = r * inv_h;
-  int iv = (int)s;
+  int iv = (int)(0.5f * (float)two_inv_h * rf);
   iv = iv < 0 ? 0 : (iv >= nint ? nint - 1 : iv);
-  const double t = 2.0 * (s - (double)iv) - 1.0;
   constexpr int NC = tab_coef<double>();
   const double2 *c = (const double2 *)(tab + (size_t)iv * tab_stride<double>());
+  const double t = fma(r, two_inv_h, -c[3].y);
   double v[8];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -766,7 +786,7 @@ __device__ __forceinline__ void wave_table<double>(const double *tab, int nint, 
     for (int q = 0; q < 4; ++q) {
       const double2 a = c[4 * p + q];
       v[2 * q] = v[2 * q] * t + a.x;
-      v[2 * q + 1] = v[2 * q + 1] * t + a.y;
+      if (q < 3) v[2 * q + 1] = v[2 * q + 1] * t + a.y;
     }
 #pragma unroll
   for (int f = 0; f < NFUNC; ++f) w[f] = v[f];
@@ -854,15 +874,16 @@ __device__ __forceinline__ void load_packed<double>(const double *__restrict__ p
 // shuffles and its first lane writes the bead row:
 //   y_i = sum_j M_r(x_i - x_j) x_j + M_self,r x_i [+ (dU + dOm x r_i, dOm, 0)]
 template <typename T, int G>
-__global__ void __launch_bounds__(256, 4) k_realspace(
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_realspace(
     int Nt, const T *__restrict__ packed, const int *__restrict__ nbr,
     const int *__restrict__ ncnt, int cap, const double *__restrict__ x, double *__restrict__ y,
-    const T *__restrict__ tab_g, int nint, T inv_h, T L, T tilt, T a, T c8, T self_t, T self_r,
+    const T *__restrict__ tab_g, int nint, T two_inv_h, T L, T tilt, T a, T c8, T self_t, T self_r,
     T self_s, int add_constraint, const int *__restrict__ bead_body,
     const double4 *__restrict__ lever, int Nt_off, const double *__restrict__ tilt_dev) {
   if (tilt_dev) tilt = (T)*tilt_dev;  // Lees-Edwards steps: the offset in device memory
   // the radial table is staged once per (persistent) CTA in shared memory
   extern __shared__ __align__(16) unsigned char tab_raw[];
+  __shared__ T group_sum[256 / G][12];
   T *tab = (T *)tab_raw;
   {
     const int nv = nint * tab_stride<T>() * (int)sizeof(T) / 16;
@@ -886,34 +907,48 @@ __global__ void __launch_bounds__(256, 4) k_realspace(
   const int *row = nbr + (size_t)i * cap;
   const T a2 = a * a, two_a = T(2) * a;
   const T invL = T(1) / L;
-#pragma unroll 2
+  const int half_hi = sizeof(T) == 8 ? __double2hiint(0.5 * (double)L) : 0;
+  // nearest image (Lees-Edwards: across y the box is offset by tilt along x).
+  // FP64: a component below L/2 by its upper word, most of them, needs no
+  // arithmetic on the FP64 pipe, which bounds that kernel.
+  auto nearest = [&](T &d0, T &d1, T &d2) {
+    if constexpr (sizeof(T) == 8) {
+      if ((__double2hiint(d1) & 0x7fffffff) >= half_hi) {
+        const T ny = rint_t<T>(d1 * invL);
+        d0 -= ny * tilt;
+        d1 -= L * ny;
+      }
+      if ((__double2hiint(d0) & 0x7fffffff) >= half_hi) d0 -= L * rint_t<T>(d0 * invL);
+      if ((__double2hiint(d2) & 0x7fffffff) >= half_hi) d2 -= L * rint_t<T>(d2 * invL);
+    } else {
+      const T ny = rint_t<T>(d1 * invL);
+      d0 -= ny * tilt;
+      d1 -= L * ny;
+      d0 -= L * rint_t<T>(d0 * invL);
+      d2 -= L * rint_t<T>(d2 * invL);
+    }
+  };
+#pragma unroll(sizeof(T) == 4 ? 2 : 1)
   for (int k = lane; k < cnt; k += G) {
     const int j = __ldg(row + k);
     T pj[3], F[3], Lm[3], S6[6];
     load_packed<T>(packed, j, pj, F, Lm, S6);
     T d0 = pi0 - pj[0], d1 = pi1 - pj[1], d2 = pi2 - pj[2];
-    {
-      // Lees-Edwards image: across y the box is offset by tilt along x
-      const T ny = rint_t<T>(d1 * invL);
-      d0 -= ny * tilt;
-      d1 -= L * ny;
-    }
-    d0 -= L * rint_t<T>(d0 * invL);
-    d2 -= L * rint_t<T>(d2 * invL);
+    nearest(d0, d1, d2);
     const T r2 = d0 * d0 + d1 * d1 + d2 * d2;
-    const T r = sqrt_t<T>(r2);
+    const T ir = inv_sqrt<T>(r2), r = r2 * ir;
     T wv[NFUNC];
-    wave_table<T>(tab, nint, inv_h, r, wv);
+    wave_table<T>(tab, nint, two_inv_h, (float)r, r, wv);
     T ph[NFUNC];
     if (r >= two_a * T(1 - 1e-6)) {
-      free_phi<T>(T(1) / r, a2, c8, ph);
+      free_phi<T>(ir, a2, c8, ph);
 #pragma unroll
       for (int f = 0; f < NFUNC; ++f) ph[f] -= wv[f];
       pair_apply<T>(d0, d1, d2, r2, ph, F, Lm, S6, acc);
     } else {
       // overlapping beads of different bodies: the free kernel is taken at
       // separation 2a along the true direction; the wave part at the true x
-      const T sc = two_a / r;
+      const T sc = two_a * ir;
       free_phi<T>(T(1) / two_a, a2, c8, ph);
       pair_apply<T>(d0 * sc, d1 * sc, d2 * sc, two_a * two_a, ph, F, Lm, S6, acc);
 #pragma unroll
@@ -921,46 +956,63 @@ __global__ void __launch_bounds__(256, 4) k_realspace(
       pair_apply<T>(d0, d1, d2, r2, ph, F, Lm, S6, acc);
     }
   }
+  // The group's sums by halves over its two upper lane bits, then over the
+  // rest: lane q G/4 holds sums 3 q .. 3 q + 2.  The eleven row components
+  // (self term, strain coordinates, rigid-body constraint, in FP64) are then
+  // finished by eleven lanes: an FP64 instruction costs the SM the same for one
+  // lane as for 32, and on one lane per group this epilogue was some 45 of them
+  // per two beads.  With the reciprocal square root above, FP32 on 32768 beads
+  // 122 -> 115 us per application; FP64 (whose pair loop it bounds: also the
+  // image test and 128 registers instead of spilling at 64) 3.07 -> 2.75 ms.
+  T r6[6], r3[3];
+  const bool up = lane & (G / 2), mid = lane & (G / 4);
+  __syncwarp();
 #pragma unroll
-  for (int off = G / 2; off > 0; off >>= 1)
+  for (int k = 0; k < 6; ++k)
+    r6[k] = (up ? acc[k + 6] : acc[k]) + __shfl_xor_sync(0xffffffffu, up ? acc[k] : acc[k + 6], G / 2);
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], off, G);
-  if (!active || lane != 0) continue;
-  // self term and rigid-body constraint rows
-  double xi_[11];
-  const double *xr = x + (size_t)i * LDB;
+  for (int k = 0; k < 3; ++k)
+    r3[k] = (mid ? r6[k + 3] : r6[k]) + __shfl_xor_sync(0xffffffffu, mid ? r6[k] : r6[k + 3], G / 4);
 #pragma unroll
-  for (int k = 0; k < 11; ++k) xi_[k] = xr[k];
-  double o[12];
-  o[0] = (double)acc[0] + (double)self_t * xi_[0];
-  o[1] = (double)acc[1] + (double)self_t * xi_[1];
-  o[2] = (double)acc[2] + (double)self_t * xi_[2];
-  o[3] = (double)acc[3] + (double)self_r * xi_[3];
-  o[4] = (double)acc[4] + (double)self_r * xi_[4];
-  o[5] = (double)acc[5] + (double)self_r * xi_[5];
-  const double exx = acc[6], eyy = acc[7], ezz = acc[8], exy = acc[9], exz = acc[10],
-               eyz = acc[11];
-  const double r2i = 0.70710678118654752440, r6i = 0.40824829046386301637, s2 = 1.41421356237309504880;
-  o[6] = r2i * (exx - eyy) + (double)self_s * xi_[6];
-  o[7] = r6i * (2.0 * ezz - exx - eyy) + (double)self_s * xi_[7];
-  o[8] = s2 * exy + (double)self_s * xi_[8];
-  o[9] = s2 * exz + (double)self_s * xi_[9];
-  o[10] = s2 * eyz + (double)self_s * xi_[10];
-  o[11] = 0.0;
-  if (add_constraint) {
-    const int J = bead_body[i];
-    const double *u = x + Nt_off + 6 * (size_t)J;
-    const double4 rv = lever[i];
-    o[0] += u[0] + (u[4] * rv.z - u[5] * rv.y);
-    o[1] += u[1] + (u[5] * rv.x - u[3] * rv.z);
-    o[2] += u[2] + (u[3] * rv.y - u[4] * rv.x);
-    o[3] += u[3];
-    o[4] += u[4];
-    o[5] += u[5];
+  for (int off = G / 8; off > 0; off >>= 1)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r3[k] += __shfl_xor_sync(0xffffffffu, r3[k], off);
+  T *sum = group_sum[threadIdx.x / G];
+  if (lane % (G / 4) == 0) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) sum[(lane / (G / 4)) * 3 + k] = r3[k];
   }
-  double2 *yo = (double2 *)(y + (size_t)i * LDB);
-#pragma unroll
-  for (int k = 0; k < 6; ++k) yo[k] = make_double2(o[2 * k], o[2 * k + 1]);
+  __syncwarp();
+  if (active) {
+    const double *xr = x + (size_t)i * LDB;
+    for (int k = lane; k < LDB; k += G) {
+      double o = 0.0;
+      if (k < 6) {
+        o = fma((double)(k < 3 ? self_t : self_r), xr[k], (double)sum[k]);
+        if (add_constraint) {
+          const double *u = x + Nt_off + 6 * (size_t)bead_body[i];
+          o += u[k];
+          if (k < 3) {  // + omega x r
+            const double *rv = (const double *)(lever + i);
+            const int k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
+            o += u[3 + k1] * rv[k2] - u[3 + k2] * rv[k1];
+          }
+        }
+      } else if (k < 11) {
+        constexpr double r2i = 0.70710678118654752440, r6i = 0.40824829046386301637;
+        // strain coordinates of (xx, yy, zz, xy, xz, yz) = sums 6 .. 11
+        double e;
+        if (k < 8)
+          e = k == 6 ? r2i * ((double)sum[6] - (double)sum[7])
+                     : r6i * (2.0 * (double)sum[8] - (double)sum[6] - (double)sum[7]);
+        else
+          e = 2.0 * r2i * (double)sum[k + 1];
+        o = fma((double)self_s, xr[k], e);
+      }
+      y[(size_t)i * LDB + k] = o;
+    }
+  }
+  __syncwarp();
   }
 }
 
@@ -1034,7 +1086,7 @@ void launch_realspace(Ctx &c, const double *x, double *y, bool add_constraint, b
   const int G = realspace_group(c);
   const size_t smem = (size_t)c.tab_nint * tab_stride<T>() * sizeof(T);
   if (smem > 200 * 1024) throw Invalid{"real-space table too large (reduce rc or raise xi)"};
-  const T inv_h = (T)(1.0 / c.tab_h);
+  const T two_inv_h = (T)(2.0 / c.tab_h);
   const T c8 = (T)(1.0 / (8.0 * kPi * c.eta));
 #define FSD_RS_LAUNCH(GG)                                                                    \
   {                                                                                          \
@@ -1043,7 +1095,7 @@ void launch_realspace(Ctx &c, const double *x, double *y, bool add_constraint, b
     k_realspace<T, GG><<<std::min<int64_t>(ceil_div((int64_t)c.Nt * GG, threads),             \
                                            (int64_t)std::max(1, per_sm) * c.num_sms),       \
                          threads, smem, c.stream>>>(                                         \
-        c.Nt, op.packed.p, c.nbr.p, c.ncnt.p, c.cap, x, y, op.table.p, c.tab_nint, inv_h,    \
+        c.Nt, op.packed.p, c.nbr.p, c.ncnt.p, c.cap, x, y, op.table.p, c.tab_nint, two_inv_h, \
         (T)c.L, (T)c.tilt, (T)c.a, c8, op.self_real[0], op.self_real[1], op.self_real[2],  \
         add_constraint ? 1 : 0, c.bead_body.p, (const double4 *)c.lever64.p,                 \
         (int)(LDB * (int64_t)c.Nt), tilt_dev_ptr(c));                                        \
