@@ -51,6 +51,14 @@ struct ZBrown {
   double tau = 0.0, ks2 = 0.0, xi = 0.0, alpha = 0.0, a = 0.0, eta = 0.0, isv = 0.0;
 };
 
+// Velocity fields after the inverse transform: FP32 grids whose side is a
+// multiple of 4 are stored in bricks of 4 x 4 x 2 points,
+// [6][z/2][y/4][x/4][z%2][y%4][x%4] (one 128-byte line each, for the
+// interpolation), other FP32 grids as planar rows [6][z][y][x], FP64
+// interleaved [z][y][x][8].
+template <typename T, int n>
+inline constexpr bool kFftBricks = sizeof(T) == 4 && n % 4 == 0;
+
 // Launchers of one (precision, size).
 template <typename T>
 struct FftOps {
@@ -59,7 +67,6 @@ struct FftOps {
   void (*y_pass)(cudaStream_t, Cplx<T> *spec, const Cplx<T> *tw, bool inverse) = nullptr;
   void (*z_green)(cudaStream_t, Cplx<T> *spec, const Cplx<T> *tw, const ZGreen<T> &) = nullptr;
   void (*z_brown)(cudaStream_t, Cplx<T> *spec, const Cplx<T> *tw, const ZBrown<T> &) = nullptr;
-  // out: planar [6][n^3] (FP32) or interleaved [n^3][8] (FP64)
   void (*x_inv)(cudaStream_t, const Cplx<T> *spec, T *out, const Cplx<T> *tw) = nullptr;
 };
 
@@ -353,7 +360,25 @@ __global__ void __launch_bounds__(Tile<T, R1, R2>::XIT)
     }
   }
   __syncthreads();
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (kFftBricks<T, n>) {
+    // lanes take the four rows of a brick first, so that a store fills whole
+    // 64-byte halves of bricks
+    for (int b = threadIdx.x; b < 3 * X * R1; b += NT) {
+      const int r = b >> 2, k1 = r % R1, q = r / R1, l = (q % (X / 4)) * 4 + (b & 3), p = q / (X / 4);
+      if (y0 + l < n) {
+        Cplx<T> v[R2];
+        second_dft<R1, R2, 1>(v, k1, sm + (p * X + l) * L::LT);
+        T *oa = out + p * n3 + ((int64_t)(z >> 1) * (n / 4) + (y0 + l) / 4) * (8 * n) + (z & 1) * 16 + (l & 3) * 4,
+          *ob = oa + 3 * n3;
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) {
+          const int x = k1 + R1 * k2, at = (x >> 2) * 32 + (x & 3);
+          oa[at] = v[k2].x;
+          ob[at] = v[k2].y;
+        }
+      }
+    }
+  } else if constexpr (sizeof(T) == 4) {
     for (int b = threadIdx.x; b < 3 * X * R1; b += NT) {
       const int k1 = b % R1, r = b / R1, l = r % X, p = r / X;
       if (y0 + l < n) {

@@ -16,8 +16,8 @@
 // FFT.  Sizes that factor into two register DFTs (fft.cuh; every even
 // 2,3,5-smooth size up to 400 but 250 and 384) run as one pass per axis on
 // three complex fields g_p + i g_(p+3), with the Green's function between the
-// forward and inverse z transforms; the inverse leaves planar velocity fields
-// [6][n^3] (FP32) or interleaved ones [n^3][8] (FP64).  On the 32768-bead
+// forward and inverse z transforms; the inverse leaves bricked or planar velocity fields
+// (FP32) or interleaved ones [n^3][8] (FP64).  On the 32768-bead
 // benchmark (n = 144, FP32) the five passes take 0.165 ms against 0.243 for
 // the fused plane kernels and staged z pass they replaced, 0.62 against 1.31
 // ms at n = 216 and, in FP64, 0.71 against 1.08 ms at n = 96.  Other sizes
@@ -31,8 +31,8 @@
 //   u_hat = A(k) (I - kk) [fM g_F_hat + fD g_D_hat],
 //   A(k) = (1 + k^2/(4 xi^2)) exp(-k^2/(4 xi^2) + k^2/(2 alpha)) / (eta k^2),
 // read-outs: velocity from fM u_hat, rotation / strain from grad (fD u_hat)
-// (k_interp_v4 for FP32 planar fields on grids that are multiples of 4,
-// k_interp for other FP32 planar fields, k_interp_rows for interleaved
+// (k_interp_brick for FP32 grids that are multiples of 4, in bricks,
+// k_interp for other FP32 grids, planar, k_interp_rows for interleaved
 // fields: FP64 and the staged plan's).
 #include "fft.cuh"
 
@@ -1220,111 +1220,140 @@ __global__ void __launch_bounds__(256) k_interp_rows(int Nt, const typename V4Of
   yr[10] += s2 * 0.5 * (G12 + G21);
 }
 
-// FP32 interpolation from planar fields [6][n^3] (n a multiple of 4): the
-// sums of k_interp, with each lane reading an aligned quad of four x points
-// of one grid row per field (six 16-byte loads); slots outside the bead's x
-// window carry weight 0 (the quads of k_spread_v4).  The warp's items are
-// (quad, y row, z row) with a fixed quad count NQ = (P + 7) / 4 per row
-// (lanes past the bead's own quad count skip), so that the item index splits
-// with two multiply-shift divisions; the window tables hold (w, offset)
-// pairs and the rows' grid offsets, and the factor 2 alpha of the dipole
-// read-out is applied once per bead.
-__global__ void __launch_bounds__(256, 4) k_interp_v4(int Nt, const float4 *__restrict__ pos,
-                                                   const float *__restrict__ field, double *y, int n,
-                                                   int P, float h, float alpha, float cnorm_h3,
-                                                   TauArg ta_, FastDiv fq, FastDiv fp) {
-  const double tau = tau_of(ta_);
-  __shared__ float2 swy[8][2][kMaxP];  // (w, offset) of the y and z window rows
-  __shared__ int srow[8][2][kMaxP];    // grid offsets of the rows: y n, z n^2
-  __shared__ __align__(16) float sxw[8][4 * kMaxQ], sxy[8][4 * kMaxQ];
-  __shared__ int sxq[8][kMaxQ];
+// Bead-row components of the read-out from its twelve window sums (u, then the
+// gradient G_ab row by row): component k = sum of up to three coef[k][t] a[idx]
+// plus, in a Lees-Edwards box (d/dy = d/ds_y - tau d/ds_x on the sheared
+// window), tau coef[k][3] a[idx[k][3]].
+__device__ const int kReadIdx[11][4] = {{0, 0, 0, 0}, {1, 1, 1, 1}, {2, 2, 2, 2}, {10, 8, 8, 9}, {5, 9, 9, 9},
+                                        {6, 4, 4, 3}, {3, 7, 7, 6}, {11, 3, 7, 6}, {4, 6, 6, 3}, {5, 9, 9, 9},
+                                        {8, 10, 10, 9}};
+#define FSD_R2I 0.70710678118654752440
+#define FSD_R6I 0.40824829046386301637
+__device__ const double kReadCoef[11][4] = {
+    {1.0, 0.0, 0.0, 0.0}, {1.0, 0.0, 0.0, 0.0}, {1.0, 0.0, 0.0, 0.0},
+    {0.5, -0.5, 0.0, -0.5}, {0.5, -0.5, 0.0, 0.0}, {0.5, -0.5, 0.0, 0.5},
+    {FSD_R2I, -FSD_R2I, 0.0, FSD_R2I}, {2.0 * FSD_R6I, -FSD_R6I, -FSD_R6I, FSD_R6I},
+    {FSD_R2I, FSD_R2I, 0.0, -FSD_R2I}, {FSD_R2I, FSD_R2I, 0.0, 0.0}, {FSD_R2I, FSD_R2I, 0.0, -FSD_R2I}};
+#undef FSD_R2I
+#undef FSD_R6I
+
+// FP32 interpolation from bricked fields (grids whose side is a multiple of
+// 4): the sums of k_interp, one warp per bead.  A lane owns one (y, z) row of
+// four x points of one of four neighbouring bricks along x: its x and y weights
+// stay in registers, it steps through the window's bricks along z with six
+// 16-byte loads each, and a quarter of a warp request is one 128-byte line.
+// Bound by the L1 pipe and the lines it misses (about half: each point is in
+// 19 windows on average, but few of them at once): with rows of the plain [z][y][x] layout a request
+// touched eight rows of one or two lines each, twice the lines, and spent as
+// many instructions again on splitting an item index and reading weights
+// (0.170 ms per application on 32768 beads, n = 144, P = 12; 0.157 with
+// 64-byte bricks of 4 x 4 points, whose runs straddle lines; now 0.147).  The
+// warp's sums are reduced by halves (18 shuffles instead of 60) and the eleven
+// components finished by eleven lanes: an FP64 instruction costs the same for
+// one lane as for 32.
+__global__ void __launch_bounds__(256, 3) k_interp_brick(int Nt, const float4 *__restrict__ pos,
+                                                         const float *__restrict__ field, double *y,
+                                                         int n, int P, float h, float alpha,
+                                                         float cnorm_h3, TauArg ta_) {
+  __shared__ float4 zt[8][kMaxP + 2];  // z of the window's bricks: w, w (z - p_z), field offset
+  __shared__ float red[8][12];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * 8 + warp;
   if (i >= Nt) return;
   const float4 p = pos[i];
-  const int g0x = (int)floorf(p.x / h) - P / 2 + 1;
-  const int a0 = g0x >= 0 ? (g0x & ~3) : -((-g0x + 3) & ~3);
-  const int nq = (g0x - a0 + P + 3) >> 2;
-  const int NQ = (int)fq.d;
-  for (int e = lane; e < 2 * P; e += 32) {
-    const int d = e / P, k = e - d * P;
-    const float pc = d == 0 ? p.y : p.z;
-    const int g = (int)floorf(pc / h) - P / 2 + 1 + k;
-    const float yv = float(g) * h - pc;
-    swy[warp][d][k] = make_float2(expf(-alpha * yv * yv), yv);
-    const int gi = ((g % n) + n) % n;
-    srow[warp][d][k] = d == 0 ? gi * n : gi * n * n;
+  const int g0x = (int)floorf(p.x / h) - P / 2 + 1, g0y = (int)floorf(p.y / h) - P / 2 + 1;
+  const int nb = n >> 2, g0z = (int)floorf(p.z / h) - P / 2 + 1;
+  const int bz0 = g0z >> 1, nbz = ((g0z + P - 1) >> 1) - bz0 + 1;
+  if (lane < 2 * nbz) {
+    const int g = 2 * bz0 + lane, k = g - g0z;
+    const float v = float(g) * h - p.z, w = k >= 0 && k < P ? expf(-alpha * v * v) : 0.f;
+    const int gi = g < 0 ? g + n : (g >= n ? g - n : g);
+    zt[warp][lane] = make_float4(w, w * v, __int_as_float((gi >> 1) * nb * nb * 32 + (gi & 1) * 16), 0.f);
   }
-  for (int sl = lane; sl < 4 * NQ; sl += 32) {
-    const int g = a0 + sl, k = g - g0x;
-    const float yv = float(g) * h - p.x;
-    sxw[warp][sl] = (k >= 0 && k < P) ? expf(-alpha * yv * yv) : 0.f;
-    sxy[warp][sl] = yv;
-  }
-  for (int q = lane; q < NQ; q += 32) sxq[warp][q] = (((a0 + 4 * q) % n) + n) % n;
   __syncwarp();
+  const int q4 = lane >> 3, yr = lane & 3, zr = (lane >> 2) & 1;
+  const int bx0 = g0x >> 2, by0 = g0y >> 2;  // first bricks of the window
+  const int nbx = ((g0x + P - 1) >> 2) - bx0 + 1, nby = ((g0y + P - 1) >> 2) - by0 + 1;
   const int64_t n3 = (int64_t)n * n * n;
   float acc[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = 0.f;
-  const int T = P * P * NQ;
+  for (int qg = 0; qg < nbx; qg += 4) {
+    const int bx = bx0 + qg + q4;
+    const bool in = qg + q4 < nbx;
+    const int bw = bx < 0 ? bx + nb : (bx >= nb ? bx - nb : bx);
+    float xw[4], xv[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int g = 4 * bx + e, k = g - g0x;
+      const float v = float(g) * h - p.x;
+      xw[e] = in && k >= 0 && k < P ? expf(-alpha * v * v) : 0.f;
+      xv[e] = xw[e] * v;
+    }
+    for (int yb = 0; yb < nby; ++yb) {
+      const int by = by0 + yb, gy = 4 * by + yr, ky = gy - g0y;
+      if (!in || ky < 0 || ky >= P) continue;
+      const float vy = float(gy) * h - p.y, wy = expf(-alpha * vy * vy);
+      const int yw = by < 0 ? by + nb : (by >= nb ? by - nb : by);
+      const float *f0 = field + (yw * nb + bw) * 32 + yr * 4;
+      float u[3] = {0.f, 0.f, 0.f}, tx[3] = {0.f, 0.f, 0.f}, ty[3] = {0.f, 0.f, 0.f}, tz[3] = {0.f, 0.f, 0.f};
 #pragma unroll 2
-  for (int t = lane; t < T; t += 32) {
-    const int r = (int)fdiv((uint32_t)t, fq), q = t - r * NQ;
-    if (q >= nq) continue;
-    const int iz = (int)fdiv((uint32_t)r, fp), iy = r - iz * P;
-    const float2 wy = swy[warp][0][iy], wz = swy[warp][1][iz];
-    const float wyz = wy.x * wz.x, y1 = wy.y, y2 = wz.y;
-    const float *g = field + (srow[warp][1][iz] + srow[warp][0][iy] + sxq[warp][q]);
-    float4 f[6];
+      for (int k = 0; k < nbz; ++k) {
+        const float4 zk = zt[warp][2 * k + zr];
+        const float *g = f0 + __float_as_int(zk.z);
+        float4 f[6];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) f[c] = __ldg((const float4 *)(g + c * n3));
-    const float4 xw = *(const float4 *)&sxw[warp][4 * q], xy = *(const float4 *)&sxy[warp][4 * q];
-    const float W[4] = {wyz * xw.x, wyz * xw.y, wyz * xw.z, wyz * xw.w};
-    const float WY[4] = {W[0] * xy.x, W[1] * xy.y, W[2] * xy.z, W[3] * xy.w};
+        for (int c = 0; c < 6; ++c) f[c] = __ldg((const float4 *)(g + c * n3));
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-      acc[c] += W[0] * f[c].x + W[1] * f[c].y + W[2] * f[c].z + W[3] * f[c].w;
+        for (int c = 0; c < 3; ++c) {
+          u[c] += zk.x * (xw[0] * f[c].x + xw[1] * f[c].y + xw[2] * f[c].z + xw[3] * f[c].w);
+          const float4 d = f[3 + c];
+          const float s = xw[0] * d.x + xw[1] * d.y + xw[2] * d.z + xw[3] * d.w;
+          tx[c] += zk.x * (xv[0] * d.x + xv[1] * d.y + xv[2] * d.z + xv[3] * d.w);
+          ty[c] += zk.x * s;
+          tz[c] += zk.y * s;
+        }
+      }
+      const float wv = wy * vy;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const float4 d = f[3 + a];
-      const float s = W[0] * d.x + W[1] * d.y + W[2] * d.z + W[3] * d.w;
-      acc[3 + 3 * a] += WY[0] * d.x + WY[1] * d.y + WY[2] * d.z + WY[3] * d.w;  // G_a0
-      acc[4 + 3 * a] += s * y1;                                                // G_a1
-      acc[5 + 3 * a] += s * y2;                                                // G_a2
+      for (int c = 0; c < 3; ++c) {
+        acc[c] += wy * u[c];
+        acc[3 + 3 * c] += wy * tx[c];
+        acc[4 + 3 * c] += wv * ty[c];
+        acc[5 + 3 * c] += wy * tz[c];
+      }
     }
   }
-  {
-    const float ta = 2.f * alpha;
+  // halves by lane bits 4 and 3, then sums over the remaining eight lanes
+  float r6[6], r3[3];
+  const bool b4 = lane & 16, b3 = lane & 8;
+  __syncwarp();
 #pragma unroll
-    for (int k = 3; k < 12; ++k) acc[k] *= ta;
+  for (int k = 0; k < 6; ++k)
+    r6[k] = (b4 ? acc[k + 6] : acc[k]) + __shfl_xor_sync(0xffffffffu, b4 ? acc[k] : acc[k + 6], 16);
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    r3[k] = (b3 ? r6[k + 3] : r6[k]) + __shfl_xor_sync(0xffffffffu, b3 ? r6[k] : r6[k + 3], 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r3[k] += __shfl_xor_sync(0xffffffffu, r3[k], o);
+  if ((lane & 7) == 0) {
+    const float s = lane == 0 ? 1.f : 2.f * alpha;  // the gradient sums carry 2 alpha
+#pragma unroll
+    for (int k = 0; k < 3; ++k) red[warp][(lane >> 3) * 3 + k] = s * r3[k];
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], off);
-  if (lane != 0) return;
-  double a_[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) a_[k] = (double)acc[k] * (double)cnorm_h3;
-  // Lees-Edwards box: d/dy = d/ds_y - tau d/ds_x on the sheared window
-  const double G00 = a_[3], G01 = a_[4] - tau * a_[3], G02 = a_[5], G10 = a_[6],
-               G11 = a_[7] - tau * a_[6], G12 = a_[8], G20 = a_[9], G21 = a_[10] - tau * a_[9],
-               G22 = a_[11];
-  const double r2i = 0.70710678118654752440, r6i = 0.40824829046386301637,
-               s2 = 1.41421356237309504880;
-  double *yr = y + (size_t)i * LDB;
-  yr[0] += a_[0];
-  yr[1] += a_[1];
-  yr[2] += a_[2];
-  yr[3] += 0.5 * (G21 - G12);
-  yr[4] += 0.5 * (G02 - G20);
-  yr[5] += 0.5 * (G10 - G01);
-  yr[6] += r2i * (G00 - G11);
-  yr[7] += r6i * (2.0 * G22 - G00 - G11);
-  yr[8] += s2 * 0.5 * (G01 + G10);
-  yr[9] += s2 * 0.5 * (G02 + G20);
-  yr[10] += s2 * 0.5 * (G12 + G21);
+  __syncwarp();
+  if (lane < 11) {
+    const int *ix = kReadIdx[lane];
+    const double *cf = kReadCoef[lane];
+    double v = cf[0] * (double)red[warp][ix[0]];
+    if (lane > 2) v = fma(cf[1], (double)red[warp][ix[1]], v);
+    if (lane == 7) v = fma(cf[2], (double)red[warp][ix[2]], v);
+    const double tau = tau_of(ta_);
+    if (tau != 0.0) v = fma(tau * cf[3], (double)red[warp][ix[3]], v);
+    y[(size_t)i * LDB + lane] += v * (double)cnorm_h3;
+  }
 }
 
 // ------------------------------------------- grid-centric FP32 spreading
@@ -1720,11 +1749,9 @@ static void wave_tail(Ctx &c, OpData<T> &op, Cx<T> *spec, double *y) {
   const double h3 = c.h * c.h * c.h;
   const bool planar = sizeof(T) == 4 && f;
   if (planar && n % 4 == 0)
-    k_interp_v4<<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p,
-                                                         (const float *)op.gout.p, y, n, P,
-                                                         (float)h, (float)alpha, (float)(cn * h3),
-                                                         tau_arg(c), make_fastdiv((P + 7) / 4),
-                                                         make_fastdiv(P));
+    k_interp_brick<<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p,
+                                                            (const float *)op.gout.p, y, n, P, (float)h,
+                                                            (float)alpha, (float)(cn * h3), tau_arg(c));
   else if (planar)
     k_interp<T, true><<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, posp<T>(c), op.gout.p, y, n, P,
                                                               h, alpha, (T)(cn * h3), tau_arg(c));
@@ -2171,8 +2198,7 @@ extern "C" fsd_status fsd_apply_wave_noalloc(int64_t n_beads, const double *bead
   f->x_inv(st, sp, gout, twc);
   const float cnh3 = (float)(cn * h * h * h);
   if (n % 4 == 0)
-    k_interp_v4<<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3, TauArg(),
-                                              make_fastdiv((P + 7) / 4), make_fastdiv(P));
+    k_interp_brick<<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3, TauArg());
   else
     k_interp<float, true><<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3,
                                                        TauArg());
