@@ -13,24 +13,27 @@ namespace fsd {
 constexpr int kDotBlocks = kDotPartials;
 constexpr int kDotChunk = 16;        // basis vectors per pass
 
-// partial[j * nb + blk] = sum over this block's grid-stride slice of V_j . w
+// partial[j * nb + blk] = sum over this block's grid-stride slice of V_j . w;
+// C: vectors per pass (1 for a norm: the warp reductions of the others would
+// be most of its FP64 work)
+template <int C>
 __global__ void __launch_bounds__(256) k_dot_partial(const double *__restrict__ V, int64_t ld,
                                                      int k0, int kc, const double *__restrict__ w,
                                                      int64_t n, double *partial) {
-  double acc[kDotChunk];
+  double acc[C];
 #pragma unroll
-  for (int j = 0; j < kDotChunk; ++j) acc[j] = 0.0;
+  for (int j = 0; j < C; ++j) acc[j] = 0.0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const double wi = w[i];
 #pragma unroll
-    for (int j = 0; j < kDotChunk; ++j)
+    for (int j = 0; j < C; ++j)
       if (j < kc) acc[j] += V[(int64_t)(k0 + j) * ld + i] * wi;
   }
-  __shared__ double red[kDotChunk][8];
+  __shared__ double red[C][8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int j = 0; j < kDotChunk; ++j) {
+  for (int j = 0; j < C; ++j) {
     double v = acc[j];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -67,7 +70,10 @@ void dot_multi(Ctx &c, const double *V, int64_t ld, int k, const double *w, doub
   const int64_t n = c.nunk;
   for (int k0 = 0; k0 < k; k0 += kDotChunk) {
     int kc = std::min(kDotChunk, k - k0);
-    k_dot_partial<<<kDotBlocks, 256, 0, c.stream>>>(V, ld, k0, kc, w, n, c.partial.p);
+    if (kc == 1)
+      k_dot_partial<1><<<kDotBlocks, 256, 0, c.stream>>>(V, ld, k0, kc, w, n, c.partial.p);
+    else
+      k_dot_partial<kDotChunk><<<kDotBlocks, 256, 0, c.stream>>>(V, ld, k0, kc, w, n, c.partial.p);
     FSD_LAUNCHED(c);
   }
   k_dot_final<<<k, 256, 0, c.stream>>>(c.partial.p, kDotBlocks, k, nullptr, 0, out_dev);
@@ -79,15 +85,20 @@ void dot_multi(Ctx &c, const double *V, int64_t ld, int k, const double *w, doub
 //   MODE 0:  partial dots  V_j . w
 //   MODE 1:  w -= sum_j coef_j V_j, then partial dots V_j . w
 //   MODE 2:  w -= sum_j coef_j V_j, then partial ||w||^2
-// Each thread owns up to kE elements spaced by the grid's thread count
-// (coalesced); basis vectors are taken four at a time so that 4 kE loads are
+// Each thread owns up to E elements spaced by the grid's thread count
+// (coalesced); basis vectors are taken four at a time so that 4 E loads are
 // in flight per thread; block partials go to partial[j * blocks + block] and
 // the last block to finish reduces them into out (fixed reduction order
-// throughout).  The grid is a whole number of waves over the SMs (two blocks
-// per SM on the benchmark's 417 792 unknowns), so that every SM carries the
-// same share of the FP64 multiply-adds that bound these passes; six elements
-// per thread keep the warp reductions of the dot products (1.5 FP64 adds per
-// basis vector and warp) small beside the 6 multiply-adds they sum.
+// throughout).  The FP64 pipe bounds these passes, so every SM has to carry the
+// same share of the multiply-adds, and the warp reductions of the dot products
+// (1.5 FP64 adds per basis vector and warp) have to stay small beside the E
+// multiply-adds they sum; the last block's reduction is a serial tail that
+// grows with the number of blocks.  E is the smallest of kEs whose grid fits
+// one block per SM, and 6 in whole waves beyond that.  With a fixed E = 6 the
+// 102 000 unknowns of an 8000-bead suspension kept 67 SMs busy: its Krylov
+// kernels took 6.6 ms per Brownian step and 3.4 ms per FP64 solve of 4096
+// beads, now 5.2 and 2.6; two to four blocks per SM of 128 or 256 threads, or
+// E = 8 and 12, were slower at every size.
 //
 // The basis element type B is double (the FP64 solve and the Lanczos square
 // roots: every product and sum in FP64) or float (the inner GMRES of the
@@ -96,7 +107,8 @@ void dot_multi(Ctx &c, const double *V, int64_t ld, int k, const double *w, doub
 // numbers would need FP64, whose rate is 1/74 of FP32 on this part), the
 // update sum_j coef_j V_j is formed in FP32 and subtracted from the FP64 w,
 // and the cross-warp sums stay FP64.
-constexpr int kE = 6;
+constexpr int kCT = 256;  // threads per block
+constexpr int kCW = kCT / 32;
 
 // Warp sums of four values with six shuffles: after the exchange across
 // lane bit 4 each lane keeps two of the four partial sums, after bit 3 one;
@@ -115,15 +127,15 @@ __device__ __forceinline__ R warp_sum4(const R a[4], int lane) {
   return c;
 }
 
-template <int MODE, typename B>
-__global__ void __launch_bounds__(256) k_cgs(const B *__restrict__ V, int64_t ld, int k,
+template <int MODE, typename B, int kE>
+__global__ void __launch_bounds__(kCT) k_cgs(const B *__restrict__ V, int64_t ld, int k,
                                              const int *k_dev, int k_add, double *w,
                                              const double *__restrict__ coef, int64_t n,
                                              double *partial, double *out, unsigned *ticket) {
   constexpr bool f64 = sizeof(B) == 8;
   if (k_dev) k = *k_dev + k_add;
   __shared__ B cs[kMaxBasis];
-  __shared__ double wred[kMaxBasis][8];  // per basis vector, per warp
+  __shared__ double wred[kMaxBasis][kCW];  // per basis vector, per warp
   __shared__ int last;
   // FP64: the update is a chain of fused multiply-adds with -coef (no
   // separate products and sums on the FP64 pipe, which bounds these passes)
@@ -236,7 +248,7 @@ __global__ void __launch_bounds__(256) k_cgs(const B *__restrict__ V, int64_t ld
   if (threadIdx.x < kr) {
     double s = 0.0;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) s += wred[threadIdx.x][q];
+    for (int q = 0; q < kCW; ++q) s += wred[threadIdx.x][q];
     partial[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = s;
     __threadfence();
   }
@@ -245,7 +257,7 @@ __global__ void __launch_bounds__(256) k_cgs(const B *__restrict__ V, int64_t ld
   __syncthreads();
   if (!last) return;
   const int nb = (int)gridDim.x;
-  for (int jj = warp; jj < kr; jj += 8) {
+  for (int jj = warp; jj < kr; jj += kCW) {
     // two independent sums per lane (a dependent FP64 add is long on this
     // part), in an order fixed by the grid size
     const double *pj = partial + (int64_t)jj * nb;
@@ -264,12 +276,30 @@ __global__ void __launch_bounds__(256) k_cgs(const B *__restrict__ V, int64_t ld
   if (threadIdx.x == 0) atomicExch(ticket, 0u);
 }
 
-// enough blocks for kE elements per thread, rounded up to whole waves of
-// the SMs once there are more blocks than SMs
+constexpr int kEs[] = {1, 2, 3, 4, 6};
+static int cgs_elems(int64_t n, int nsm) {
+  for (int e : kEs)
+    if (ceil_div(n, (int64_t)kCT * e) <= nsm) return e;
+  return 6;
+}
+
+// enough blocks for the elements per thread, rounded up to whole waves of the
+// SMs once there are more blocks than SMs
 static int cgs_blocks(int64_t n, int nsm) {
-  const int64_t b = std::max<int64_t>(1, ceil_div(n, 256LL * kE));
+  const int64_t b = std::max<int64_t>(1, ceil_div(n, (int64_t)kCT * cgs_elems(n, nsm)));
   if (nsm < 1 || b <= nsm) return (int)b;
   return (int)(ceil_div(b, (int64_t)nsm) * nsm);
+}
+
+template <typename B, int E>
+static void cgs_go(cudaStream_t st, int blocks, int mode, const B *V, int64_t ld, int k, const int *k_dev,
+                   int k_add, double *w, const double *coef, int64_t n, double *pp, double *out, unsigned *tk) {
+  if (mode == 0)
+    k_cgs<0, B, E><<<blocks, kCT, 0, st>>>(V, ld, k, k_dev, k_add, w, coef, n, pp, out, tk);
+  else if (mode == 1)
+    k_cgs<1, B, E><<<blocks, kCT, 0, st>>>(V, ld, k, k_dev, k_add, w, coef, n, pp, out, tk);
+  else
+    k_cgs<2, B, E><<<blocks, kCT, 0, st>>>(V, ld, k, k_dev, k_add, w, coef, n, pp, out, tk);
 }
 
 // out[j] = V_j . w (j < k); mode 1 / 2 first apply w -= V coef (mode 2:
@@ -285,12 +315,15 @@ static void cgs_launch(Ctx &c, int mode, const B *V, int64_t ld, int k, const in
   const int blocks = cgs_blocks(n, c.num_sms);
   unsigned *tk = c.cgs_ticket.p;
   double *pp = c.partial.p;
-  if (mode == 0)
-    k_cgs<0, B><<<blocks, 256, 0, c.stream>>>(V, ld, k, k_dev, k_add, w, coef_dev, n, pp, out_dev, tk);
-  else if (mode == 1)
-    k_cgs<1, B><<<blocks, 256, 0, c.stream>>>(V, ld, k, k_dev, k_add, w, coef_dev, n, pp, out_dev, tk);
-  else
-    k_cgs<2, B><<<blocks, 256, 0, c.stream>>>(V, ld, k, k_dev, k_add, w, coef_dev, n, pp, out_dev, tk);
+#define FSD_CGS(E) cgs_go<B, E>(c.stream, blocks, mode, V, ld, k, k_dev, k_add, w, coef_dev, n, pp, out_dev, tk)
+  switch (cgs_elems(n, c.num_sms)) {
+    case 1: FSD_CGS(1); break;
+    case 2: FSD_CGS(2); break;
+    case 3: FSD_CGS(3); break;
+    case 4: FSD_CGS(4); break;
+    default: FSD_CGS(6); break;
+  }
+#undef FSD_CGS
   FSD_LAUNCHED(c);
   FSD_CUDA(cudaGetLastError());
 }
