@@ -30,9 +30,10 @@ struct alignas(2 * sizeof(T)) Cplx {
   T x, y;
 };
 
-// Green's function operands of the z pass.  Cubic box: green[3 m] by
-// m = kx^2 + ky^2 + kz^2.  Lees-Edwards box: gle[kx <= n/2][kz][ky][3] for the
-// current offset, the physical wave vector (kx, ky - tau kx, kz).
+// Green's function operands of the z pass: the halved factors and 1/k^2 (in
+// (2 pi / L)^2).  Cubic box: green[4 m] by m = kx^2 + ky^2 + kz^2.  Lees-Edwards
+// box: gle[kx <= n/2][kz][ky][4] for the current offset, the physical wave vector
+// (kx, ky - tau kx, kz).
 template <typename T>
 struct ZGreen {
   const T *green = nullptr;
@@ -447,7 +448,7 @@ __global__ void __launch_bounds__(Tile<T, R1, R2>::XT)
 // u = A(k) (I - kk) [..] for one wave vector: factors t (halved: the inputs
 // are the unhalved sums gF = Z_k + conj Z_-k, gD = (Z_k - conj Z_-k) / i).
 template <typename T>
-__device__ __forceinline__ void green_apply(const T t[3], const T kk[3], T im, const Cplx<T> *gF,
+__device__ __forceinline__ void green_apply(const T t[4], const T kk[3], const Cplx<T> *gF,
                                             const Cplx<T> *gD, Cplx<T> *uM, Cplx<T> *uD) {
   Cplx<T> sF = {T(0), T(0)}, sD = {T(0), T(0)};
 #pragma unroll
@@ -457,8 +458,8 @@ __device__ __forceinline__ void green_apply(const T t[3], const T kk[3], T im, c
     sD.x += kk[d] * gD[d].x;
     sD.y += kk[d] * gD[d].y;
   }
-  sF = {sF.x * im, sF.y * im};
-  sD = {sD.x * im, sD.y * im};
+  sF = {sF.x * t[3], sF.y * t[3]};
+  sD = {sD.x * t[3], sD.y * t[3]};
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const Cplx<T> pF = {gF[d].x - kk[d] * sF.x, gF[d].y - kk[d] * sF.y};
@@ -470,27 +471,18 @@ __device__ __forceinline__ void green_apply(const T t[3], const T kk[3], T im, c
 
 __device__ __forceinline__ int signed_k(int i, int n) { return i <= n / 2 ? i : i - n; }
 
-// wave vector, 1 / k^2 and halved Green factors at grid index (kx <= n/2, y, z)
+// halved Green factors and 1 / k^2 at grid index (kx <= n/2, y, z)
 template <typename T, int n>
-__device__ __forceinline__ void green_at(const ZGreen<T> &g, double tau, int kx, int y, int z, T t[3],
-                                         T kk[3], T &im) {
+__device__ __forceinline__ void green_at(const ZGreen<T> &g, int kx, int y, int z, T t[4]) {
   const int ky = signed_k(y, n), kz = signed_k(z, n);
-  kk[0] = (T)kx;
-  kk[2] = (T)kz;
-  const T *q;
-  if (!g.gle) {
-    const int m = kx * kx + ky * ky + kz * kz;
-    q = g.green + 3 * m;
-    kk[1] = (T)ky;
-    im = T(1) / (T)m;
+  const T *q = g.gle ? g.gle + 4 * (((int64_t)kx * n + z) * n + y) : g.green + 4 * (kx * kx + ky * ky + kz * kz);
+  if constexpr (sizeof(T) == 4) {
+    const float4 v = __ldg((const float4 *)q);
+    t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
   } else {
-    const double kyp = (double)ky - tau * (double)kx;
-    q = g.gle + 3 * (((int64_t)kx * n + z) * n + y);
-    kk[1] = (T)kyp;
-    im = (T)(1.0 / ((double)(kx * kx + kz * kz) + kyp * kyp));
+    const double2 u = __ldg((const double2 *)q), v = __ldg((const double2 *)q + 1);
+    t[0] = u.x; t[1] = u.y; t[2] = v.x; t[3] = v.y;
   }
-#pragma unroll
-  for (int e = 0; e < 3; ++e) t[e] = T(0.5) * q[e];
 }
 
 // random field (I - kk) xi(k) (c fM, c fD) at grid index (kx <= n/2, y, z)
@@ -612,12 +604,21 @@ __global__ void __launch_bounds__(Tile<T, R1, R2>::ZT)
     }
     __syncthreads();
   }
-  const double tau = !BROWN && g.gle ? (g.tilt_dev ? *g.tilt_dev * g.invL : g.tau) : 0.0;
-  for (int e = threadIdx.x; e < TP * n; e += NT) {
-    const int t = e % TP, q = e / TP, k1 = q % R1, k2 = q / R1, kz = k1 + R1 * k2;
-    const int ky = ky0 + t;
-    if (ky >= kend) continue;
-    const int my = ky == 0 ? 0 : n - ky, mz = kz == 0 ? 0 : n - kz;
+  // a thread keeps its ky: the physical y component (FP64, rounded once) is
+  // found once, and 1 / k^2 comes with the factors: in FP32 these few FP64
+  // operations per point were a fifth of the pass in a Lees-Edwards box (n = 144:
+  // 66 -> 52 us; in FP64 1.06 -> 0.96 ms)
+  static_assert(NT % TP == 0, "a thread stays on one ky");
+  const int t = threadIdx.x % TP, ky = ky0 + t, my = ky == 0 ? 0 : n - ky;
+  T kk[3] = {(T)kx, (T)signed_k(ky, n), T(0)}, kyb = (T)signed_k(my, n);
+  if (!BROWN && g.gle) {
+    const double tau = g.tilt_dev ? *g.tilt_dev * g.invL : g.tau;
+    kk[1] = (T)((double)signed_k(ky, n) - tau * (double)kx);
+    kyb = (T)((double)signed_k(my, n) - tau * (double)kx);
+  }
+  for (int q = threadIdx.x / TP; q < n && ky < kend; q += NT / TP) {
+    const int k1 = q % R1, k2 = q / R1, kz = k1 + R1 * k2;
+    const int mz = kz == 0 ? 0 : n - kz;
     Cplx<T> *A = sm + t * L::LT + k1 * L::CS + k2;
     Cplx<T> *B = sm + (TP + t) * L::LT + (mz % R1) * L::CS + mz / R1;
     constexpr int ps = 2 * TP * L::LT;  // from field p to p + 1
@@ -640,11 +641,12 @@ __global__ void __launch_bounds__(Tile<T, R1, R2>::ZT)
       }
 #pragma unroll
       for (int d = 0; d < 3; ++d) uM[d] = uD[d] = {T(0), T(0)};
-      T tf[3], kk[3], im;
+      T tf[4];
       const bool zero = (kx | ky | kz) == 0;
+      kk[2] = (T)signed_k(kz, n);
       if (!zero) {
-        green_at<T, n>(g, tau, kx, ky, kz, tf, kk, im);
-        green_apply<T>(tf, kk, im, gF, gD, uM, uD);
+        green_at<T, n>(g, kx, ky, kz, tf);
+        green_apply<T>(tf, kk, gF, gD, uM, uD);
       }
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
@@ -657,8 +659,9 @@ __global__ void __launch_bounds__(Tile<T, R1, R2>::ZT)
           gF[d].y = -gF[d].y;
           gD[d].y = -gD[d].y;
         }
-        green_at<T, n>(g, tau, kx, my, mz, tf, kk, im);
-        green_apply<T>(tf, kk, im, gF, gD, vM, vD);
+        const T kb[3] = {kk[0], kyb, (T)signed_k(mz, n)};
+        green_at<T, n>(g, kx, my, mz, tf);
+        green_apply<T>(tf, kb, gF, gD, vM, vD);
       }
     }
 #pragma unroll
