@@ -158,21 +158,21 @@ static const double *dev_in(Ctx &c, const double *p, size_t count, DBuf<double> 
 // ------------------------------------------------------------------ solver
 template <typename T>
 void apply_saddle(Ctx &c, const double *x, double *y) {
+  const double *add = nullptr;
   if (!c.overlap || c.prof) {
-    launch_realspace<T>(c, x, y, true, false);
+    launch_realspace<T>(c, x, y, true);
     launch_wavespace<T>(c, x, y);
   } else {
     // the real-space sum on the second stream, the wave-space chain into yw
-    // on this one; joined before the sum and the aggregate rows (in a
-    // captured graph these are two parallel branches)
-    const int64_t nb = (int64_t)LDB * c.Nt;
+    // on this one; joined before the aggregate rows, whose kernel adds the two
+    // (in a captured graph these are two parallel branches)
     FSD_CUDA(cudaEventRecord(c.ev_fork, c.stream));
     FSD_CUDA(cudaStreamWaitEvent(c.stream2, c.ev_fork, 0));
     cudaStream_t main = c.stream;
     c.stream = c.stream2;
     c.rs_overlapped = true;
     try {
-      launch_realspace<T>(c, x, y, true, false);
+      launch_realspace<T>(c, x, y, true);
     } catch (...) {
       c.stream = main;
       c.rs_overlapped = false;
@@ -181,12 +181,11 @@ void apply_saddle(Ctx &c, const double *x, double *y) {
     c.rs_overlapped = false;
     FSD_CUDA(cudaEventRecord(c.ev_join, c.stream2));
     c.stream = main;
-    FSD_CUDA(cudaMemsetAsync(c.yw.p, 0, nb * sizeof(double), c.stream));
-    launch_wavespace<T>(c, x, c.yw.p);
+    launch_wavespace<T>(c, x, c.yw.p, true);
     FSD_CUDA(cudaStreamWaitEvent(c.stream, c.ev_join, 0));
-    launch_axpy(c, c.yw.p, y, nb);
+    add = c.yw.p;
   }
-  launch_body_rows<T>(c, x, y, true);
+  launch_body_rows<T>(c, x, y, true, add);
 }
 template void apply_saddle<float>(Ctx &, const double *, double *);
 template void apply_saddle<double>(Ctx &, const double *, double *);
@@ -1326,10 +1325,10 @@ fsd_status fsd_apply_mobility(fsd_ctx *ctx, const double *in, double *out, int p
   double *y = c.t2.p;
   FSD_CUDA(cudaMemsetAsync(y, 0, c.nunk * sizeof(double), c.stream));
   if (precision == FSD_FP64) {
-    if (part & 1) launch_realspace<double>(c, c.t1.p, y, false, false);
+    if (part & 1) launch_realspace<double>(c, c.t1.p, y, false);
     if (part & 2) launch_wavespace<double>(c, c.t1.p, y);
   } else {
-    if (part & 1) launch_realspace<float>(c, c.t1.p, y, false, false);
+    if (part & 1) launch_realspace<float>(c, c.t1.p, y, false);
     if (part & 2) launch_wavespace<float>(c, c.t1.p, y);
   }
   vec_out(c, y, out, true, false);

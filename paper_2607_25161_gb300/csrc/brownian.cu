@@ -343,9 +343,9 @@ void brownian_sample(Ctx &c, double kT, double dt, uint64_t seed, uint64_t step,
   FSD_CUDA(cudaGetLastError());
   auto real_op = [&](const double *x, double *y) {
     if (f32)
-      launch_realspace<float>(c, x, y, false, false);
+      launch_realspace<float>(c, x, y, false);
     else
-      launch_realspace<double>(c, x, y, false, false);
+      launch_realspace<double>(c, x, y, false);
   };
   double ch_r = 0.0, ch_n = 0.0;
   const int ir = lanczos_sqrt(c, real_op, c.bwork.p, c.t2.p, tol, maxit, &ch_r);

@@ -308,8 +308,7 @@ __device__ inline void philox_normals4(uint64_t seed, uint64_t step, uint32_t st
 void build_real_table(Ctx &c);
 void build_neighbors(Ctx &c);  // cell list + mobility and lubrication lists
 template <typename T>
-void launch_realspace(Ctx &c, const double *x, double *y, bool add_constraint,
-                      bool self_only_real);
+void launch_realspace(Ctx &c, const double *x, double *y, bool add_constraint);
 void launch_wrap_positions(Ctx &c);  // pos64 / op*.pos / levers from X, q, rbody
 __global__ void k_exclusive_scan(int n, const int *__restrict__ in, int *out, int *cursor);
 __global__ void __launch_bounds__(128) k_sort_cells(int ncells, const int *__restrict__ cell_start,
@@ -333,19 +332,22 @@ int realspace_group(const Ctx &c);   // lanes per bead of the pair sum
 // wavespace.cu
 void build_wave(Ctx &c);
 template <typename T>
-void launch_wavespace(Ctx &c, const double *x, double *y);  // y += M_w x
+void launch_wavespace(Ctx &c, const double *x, double *y,
+                      bool set = false);  // y += M_w x, or y = M_w x (bead rows)
 
 // nearfield.cu
 void build_lubrication(Ctx &c);  // BSR blocks (both precisions) + Schur LU
 template <typename T>
-void launch_body_rows(Ctx &c, const double *x, double *y, bool with_lub);  // y2 = Sigma B^T x1 - RR x2
+void launch_body_rows(Ctx &c, const double *x, double *y, bool with_lub,
+                      const double *add = nullptr);  // y2 = Sigma B^T x1 - RR x2; bead rows += add
 template <typename T>
 void launch_lub_apply(Ctx &c, const double *dU, double *out);  // out = RR dU
 void launch_precond(Ctx &c, const double *r, double *z);
-// the same on column *col_dev of the bases V and Z (leading dimension ld),
-// z also written to z2 (the captured Arnoldi step)
-void launch_precond_col(Ctx &c, const double *V, double *Z, int64_t ld, const int *col_dev,
-                        double *z2);
+// the captured Arnoldi step: z_j from v_j, columns j = *col_dev of the bases V
+// and Z (leading dimension ld), z_j also to z2; for j > 0 v_j is first formed as
+// *scale_dev w (the previous step's remainder)
+void launch_precond_col(Ctx &c, double *V, double *Z, int64_t ld, const int *col_dev, double *z2,
+                        const double *w, const double *scale_dev);
 void launch_rhs(Ctx &c, const double *ft_internal, double shear, double *b);
 void launch_outputs(Ctx &c, const double *x, double shear, double *vel_int,
                     double *str_int);

@@ -235,45 +235,62 @@ __global__ void k_g_put_col(B *Z, int64_t ld, double *in, const GState *s, int64
 
 // Hessenberg column j from the two Gram-Schmidt passes, the earlier Givens
 // rotations applied to it, a new rotation that zeroes h_{j+1,j}, and the
-// stopping test of the Arnoldi loop.
-__global__ void k_g_givens(GState *s, cudaGraphConditionalHandle h_arn, int is64) {
-  if (threadIdx.x | blockIdx.x) return;
+// stopping test of the Arnoldi loop.  The column and the rotations are fetched
+// and stored by 64 threads; one runs the rotations, a chain of one fused
+// multiply-add each (the other product does not wait for it), from shared
+// memory: from global memory every link also waited for its loads.
+__global__ void __launch_bounds__(64) k_g_givens(GState *s, cudaGraphConditionalHandle h_arn, int is64) {
+  static_assert(kMaxM < 64, "a thread per entry of the column");
+  __shared__ double col[64], csn[64], snn[64];
+  const int t = threadIdx.x;
   const int j = s->j, m = s->m;
   double *H = s->H;
-  for (int i = 0; i <= j; ++i) H[i * m + j] = s->h[i] + s->h[64 + i];
+  if (t <= j) col[t] = s->h[t] + s->h[64 + t];
+  if (t < j) {
+    csn[t] = s->cs[t];
+    snn[t] = s->sn[t];
+  }
+  __syncthreads();
   const double hnext = sqrt(fmax(0.0, s->h[128]));
-  if (is64)
-    s->mv64++;
-  else
-    s->mv32++;
-  if (!(hnext == hnext)) {
-    s->status |= 1;
-    s->cont = 0;
-    set_cond(h_arn, false);
-    return;
+  if (t == 0) {
+    double a = col[0];
+#pragma unroll 4
+    for (int i = 0; i < j; ++i) {
+      const double b = col[i + 1], c = csn[i], d = snn[i];
+      col[i] = fma(c, a, d * b);
+      a = fma(-d, a, c * b);
+    }
+    const double den = hypot(a, hnext);
+    const double cj = den > 0 ? a / den : 1.0, sj = den > 0 ? hnext / den : 0.0;
+    col[j] = den;
+    if (is64)
+      s->mv64++;
+    else
+      s->mv32++;
+    if (!(hnext == hnext)) {
+      s->status |= 1;
+      s->cont = 0;
+      set_cond(h_arn, false);
+    } else {
+      s->cs[j] = cj;
+      s->sn[j] = sj;
+      const double g = s->g[j], r = -sj * g;
+      s->g[j + 1] = r;
+      s->g[j] = cj * g;
+      const double resid = fabs(r);
+      s->resid = resid;
+      s->j = j + 1;
+      s->total++;
+      s->cyc_total++;
+      const bool stop = resid <= s->stoptol || hnext <= 1e-300 || s->j >= m ||
+                        s->total >= s->max_total || s->cyc_total >= s->cyc_max;
+      s->cont = stop ? 0 : 1;
+      s->scale = stop ? 0.0 : 1.0 / hnext;
+      set_cond(h_arn, !stop);
+    }
   }
-  for (int i = 0; i < j; ++i) {
-    const double a = H[i * m + j], b = H[(i + 1) * m + j];
-    H[i * m + j] = s->cs[i] * a + s->sn[i] * b;
-    H[(i + 1) * m + j] = -s->sn[i] * a + s->cs[i] * b;
-  }
-  const double a = H[j * m + j];
-  const double den = hypot(a, hnext);
-  s->cs[j] = den > 0 ? a / den : 1.0;
-  s->sn[j] = den > 0 ? hnext / den : 0.0;
-  H[j * m + j] = den;
-  s->g[j + 1] = -s->sn[j] * s->g[j];
-  s->g[j] = s->cs[j] * s->g[j];
-  const double resid = fabs(s->g[j + 1]);
-  s->resid = resid;
-  s->j = j + 1;
-  s->total++;
-  s->cyc_total++;
-  const bool stop = resid <= s->stoptol || hnext <= 1e-300 || s->j >= m ||
-                    s->total >= s->max_total || s->cyc_total >= s->cyc_max;
-  s->cont = stop ? 0 : 1;
-  s->scale = stop ? 0.0 : 1.0 / hnext;
-  set_cond(h_arn, !stop);
+  __syncthreads();
+  if (t <= j) H[t * m + j] = col[t];
 }
 
 // V_j = w / h_{j,j-1} when the loop goes on
@@ -375,8 +392,9 @@ static void arnoldi_step(Ctx &c, GState *s, cudaGraphConditionalHandle h_arn) {
   B *V = basis_v(c, B()), *Z = basis_z(c, B());
   if constexpr (sizeof(B) == 8) {
     // z_j = P^-1 v_j straight from and into the bases (column j read on the
-    // device), and into the operator's fixed input buffer
-    launch_precond_col(c, V, Z, ld, &s->j, gc.zf.p);
+    // device; v_j formed here from the last step's remainder), and into the
+    // operator's fixed input buffer
+    launch_precond_col(c, V, Z, ld, &s->j, gc.zf.p, c.w.p, &s->scale);
   } else {
     k_g_get_col<B><<<nb, 256, 0, c.stream>>>(gc.vin.p, V, ld, s, n);
     FSD_LAUNCHED(c);
@@ -388,10 +406,12 @@ static void arnoldi_step(Ctx &c, GState *s, cudaGraphConditionalHandle h_arn) {
   cgs_pass_dev(c, 0, V, ld, &s->j, 1, mm, c.w.p, nullptr, s->h);
   cgs_pass_dev(c, 1, V, ld, &s->j, 1, mm, c.w.p, s->h, s->h + 64);
   cgs_pass_dev(c, 2, V, ld, &s->j, 1, mm, c.w.p, s->h + 64, s->h + 128);
-  k_g_givens<<<1, 32, 0, c.stream>>>(s, h_arn, sizeof(T) == 8 ? 1 : 0);
+  k_g_givens<<<1, 64, 0, c.stream>>>(s, h_arn, sizeof(T) == 8 ? 1 : 0);
   FSD_LAUNCHED(c);
-  k_g_next_col<B><<<nb, 256, 0, c.stream>>>(V, ld, c.w.p, s, n);
-  FSD_LAUNCHED(c);
+  if constexpr (sizeof(B) == 4) {
+    k_g_next_col<B><<<nb, 256, 0, c.stream>>>(V, ld, c.w.p, s, n);
+    FSD_LAUNCHED(c);
+  }
   FSD_CUDA(cudaGetLastError());
 }
 

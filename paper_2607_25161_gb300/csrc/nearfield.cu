@@ -338,6 +338,9 @@ __global__ void __launch_bounds__(128) k_schur_lu(int N, const int *__restrict__
       for (int cc = k + 1; cc < 6; ++cc) Bm[6 * rr + cc] -= f * Bm[6 * k + cc];
     }
   }
+  // the solves divide by the diagonal: stored inverted
+#pragma unroll
+  for (int k = 0; k < 6; ++k) Bm[7 * k] = 1.0 / Bm[7 * k];
 #pragma unroll
   for (int e = 0; e < 36; ++e) schur[(size_t)J * 36 + e] = Bm[e];
 #pragma unroll
@@ -357,7 +360,7 @@ __device__ __forceinline__ void lu_solve6(const double *LU, const int *pv, doubl
     for (int k = 0; k < a; ++k) v[a] -= LU[6 * a + k] * v[k];
   for (int a = 5; a >= 0; --a) {
     for (int k = a + 1; k < 6; ++k) v[a] -= LU[6 * a + k] * v[k];
-    v[a] /= LU[6 * a + a];
+    v[a] *= LU[6 * a + a];  // stored inverted
   }
 }
 
@@ -369,19 +372,27 @@ __device__ __forceinline__ void lu_solve6(const double *LU, const int *pv, doubl
 // then write the bead rows z1 of their beads from z2 held in registers.
 // With col_dev non-null, r and z are column *col_dev of bases with leading
 // dimension ld (the captured Arnoldi step, whose column index lives on the
-// device), and z is also written to z2.
+// device), z is also written to z2, and for a column past the first r is formed
+// as *scale w and stored: the basis vector's scaling rides along.
 template <int LPA>
-__global__ void __launch_bounds__(256) k_precond(int N, const int *__restrict__ body_start,
-                                                 const double4 *__restrict__ lever,
-                                                 const double *__restrict__ r, double *z,
-                                                 const double *__restrict__ schur,
-                                                 const int *__restrict__ piv, double zeta0,
-                                                 int64_t off, const int *col_dev, int64_t ld,
-                                                 double *z2) {
+__global__ void __launch_bounds__(256) k_precond(
+    int N, const int *__restrict__ body_start, const double4 *__restrict__ lever, double *r_,
+    double *z, const double *__restrict__ schur, const int *__restrict__ piv, double zeta0,
+    int64_t off, const int *col_dev, int64_t ld, double *z2, const double *__restrict__ w,
+    const double *scale) {
+  double *keep = nullptr;  // where r is stored
+  double sc = 1.0;
+  const double *r = r_;
   if (col_dev) {
-    const int64_t o = (int64_t)*col_dev * ld;
+    const int col = *col_dev;
+    const int64_t o = (int64_t)col * ld;
     r += o;
     z += o;
+    if (w && col > 0) {
+      keep = r_ + o;
+      r = w;
+      sc = *scale;
+    }
   }
   const int J = (blockIdx.x * blockDim.x + threadIdx.x) / LPA;
   const int sub = threadIdx.x & (LPA - 1);
@@ -404,7 +415,11 @@ __global__ void __launch_bounds__(256) k_precond(int N, const int *__restrict__ 
     for (int k = 0; k < 6; ++k) g[k] += __shfl_xor_sync(0xffffffffu, g[k], o);
   if (!active) return;
   double v[6];
-  for (int k = 0; k < 6; ++k) v[k] = r[off + 6 * (size_t)J + k] - zeta0 * g[k];
+  for (int k = 0; k < 6; ++k) {
+    const double rk = sc * r[off + 6 * (size_t)J + k];
+    if (keep && sub == 0) keep[off + 6 * (size_t)J + k] = rk;
+    v[k] = rk - zeta0 * (sc * g[k]);
+  }
   lu_solve6(schur + (size_t)J * 36, piv + 6 * J, v);
   // u = z2 = -v
   if (sub == 0)
@@ -414,21 +429,36 @@ __global__ void __launch_bounds__(256) k_precond(int N, const int *__restrict__ 
     }
   for (int b = b0 + sub; b < b1; b += LPA) {
     const double4 rv = lever[b];
-    const double *ri = r + (size_t)b * LDB;
-    double zo[LDB];
+    double ri[LDB], zo[LDB];
+    const double2 *src = (const double2 *)(r + (size_t)b * LDB);
+#pragma unroll
+    for (int k = 0; k < LDB / 2; ++k) {
+      const double2 t = src[k];
+      ri[2 * k] = t.x;
+      ri[2 * k + 1] = t.y;
+    }
+    if (keep) {
+      double2 *kp = (double2 *)(keep + (size_t)b * LDB);
+#pragma unroll
+      for (int k = 0; k < LDB; ++k) ri[k] *= sc;
+#pragma unroll
+      for (int k = 0; k < LDB / 2; ++k) kp[k] = make_double2(ri[2 * k], ri[2 * k + 1]);
+    }
     zo[0] = zeta0 * (ri[0] + (v[0] + v[4] * rv.z - v[5] * rv.y));
     zo[1] = zeta0 * (ri[1] + (v[1] + v[5] * rv.x - v[3] * rv.z));
     zo[2] = zeta0 * (ri[2] + (v[2] + v[3] * rv.y - v[4] * rv.x));
     zo[3] = zeta0 * (ri[3] + v[3]);
     zo[4] = zeta0 * (ri[4] + v[4]);
     zo[5] = zeta0 * (ri[5] + v[5]);
+#pragma unroll
     for (int k = 6; k < 11; ++k) zo[k] = zeta0 * ri[k];
     zo[11] = 0.0;
-    double *zi = z + (size_t)b * LDB;
-    for (int k = 0; k < LDB; ++k) zi[k] = zo[k];
-    if (z2) {
-      double *zj = z2 + (size_t)b * LDB;
-      for (int k = 0; k < LDB; ++k) zj[k] = zo[k];
+    double2 *zi = (double2 *)(z + (size_t)b * LDB), *zj = (double2 *)(z2 + (size_t)b * LDB);
+#pragma unroll
+    for (int k = 0; k < LDB / 2; ++k) {
+      const double2 t = make_double2(zo[2 * k], zo[2 * k + 1]);
+      zi[k] = t;
+      if (z2) zj[k] = t;
     }
   }
 }
@@ -454,7 +484,25 @@ __global__ void __launch_bounds__(256) k_body_rows(
     int N, const int *__restrict__ body_start, const int *__restrict__ bead_body,
     const typename LV<T>::type *__restrict__ lever, const double *__restrict__ x, double *y,
     const int *__restrict__ brow, const int *__restrict__ bcol, const T *__restrict__ bval,
-    const T *__restrict__ bdiag, int with_lub, int64_t off, T sgn_bead, T sgn_lub) {
+    const T *__restrict__ bdiag, int with_lub, int64_t off, T sgn_bead, T sgn_lub,
+    const double *__restrict__ add) {
+  // the blocks past the aggregates': bead rows += add (the wave-space part of an
+  // overlapped application), 256 threads x 2 pairs each
+  if ((int64_t)blockIdx.x * blockDim.x >= (int64_t)N * LPA) {
+    const int first = (N * LPA + 255) / 256;
+    double2 *o = (double2 *)y;
+    const double2 *q = (const double2 *)add;
+    const int64_t n2 = off / 2, e0 = ((int64_t)blockIdx.x - first) * 512 + threadIdx.x;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int64_t e = e0 + 256 * u;
+      if (e < n2) {
+        const double2 a = o[e], b = q[e];
+        o[e] = make_double2(a.x + b.x, a.y + b.y);
+      }
+    }
+    return;
+  }
   const int J = (blockIdx.x * blockDim.x + threadIdx.x) / LPA;
   const int sub = threadIdx.x & (LPA - 1);
   const bool active = J < N;
@@ -1008,13 +1056,15 @@ OpData<float> &opx<float>(Ctx &c) {
 }
 
 template <typename T>
-static void body_rows_launch(Ctx &c, const double *x, double *y, int lub, T sgn_bead, T sgn_lub) {
+static void body_rows_launch(Ctx &c, const double *x, double *y, int lub, T sgn_bead, T sgn_lub,
+                             const double *add = nullptr) {
   OpData<T> &op = opx<T>(c);
   const int64_t off = (int64_t)LDB * c.Nt;
+  const int extra = add ? ceil_div(off / 2, 512) : 0;
 #define FSD_BODY_ROWS(LPA)                                                                      \
-  k_body_rows<T, LPA><<<ceil_div((int64_t)c.N * LPA, 256), 256, 0, c.stream>>>(                \
+  k_body_rows<T, LPA><<<ceil_div((int64_t)c.N * LPA, 256) + extra, 256, 0, c.stream>>>(        \
       c.N, c.body_start.p, c.bead_body.p, lever_ptr<T>(c), x, y, c.brow.p, c.bcol.p, op.bval.p, \
-      op.bdiag.p, lub, off, sgn_bead, sgn_lub)
+      op.bdiag.p, lub, off, sgn_bead, sgn_lub, add)
   switch (c.body_lanes) {
     case 4: FSD_BODY_ROWS(4); break;
     case 8: FSD_BODY_ROWS(8); break;
@@ -1025,10 +1075,10 @@ static void body_rows_launch(Ctx &c, const double *x, double *y, int lub, T sgn_
 }
 
 template <typename T>
-void launch_body_rows(Ctx &c, const double *x, double *y, bool with_lub) {
+void launch_body_rows(Ctx &c, const double *x, double *y, bool with_lub, const double *add) {
   ProfScope ps(c, PG_BODY);
   const bool lub = with_lub && c.n_lub > 0;
-  body_rows_launch<T>(c, x, y, lub ? 1 : 0, T(1), T(-1));
+  body_rows_launch<T>(c, x, y, lub ? 1 : 0, T(1), T(-1), add);
   FSD_LAUNCHED(c);
   FSD_CUDA(cudaGetLastError());
 }
@@ -1042,15 +1092,15 @@ void launch_lub_apply(Ctx &c, const double *x, double *y) {
   FSD_CUDA(cudaGetLastError());
 }
 
-static void precond_launch(Ctx &c, const double *r, double *z, const int *col_dev, int64_t ld,
-                           double *z2) {
+static void precond_launch(Ctx &c, double *r, double *z, const int *col_dev, int64_t ld, double *z2,
+                           const double *w, const double *scale) {
   ProfScope ps(c, PG_PRECOND);
   const int64_t off = (int64_t)LDB * c.Nt;
   const double zeta0 = 6.0 * kPi * c.eta * c.a;
-#define FSD_PRECOND(LPA)                                                                  \
-  k_precond<LPA><<<ceil_div((int64_t)c.N * LPA, 256), 256, 0, c.stream>>>(                \
+#define FSD_PRECOND(LPA)                                                                      \
+  k_precond<LPA><<<ceil_div((int64_t)c.N * LPA, 256), 256, 0, c.stream>>>(                    \
       c.N, c.body_start.p, (const double4 *)c.lever64.p, r, z, c.schur.p, c.piv.p, zeta0, off, \
-      col_dev, ld, z2)
+      col_dev, ld, z2, w, scale)
   switch (c.body_lanes) {
     case 4: FSD_PRECOND(4); break;
     case 8: FSD_PRECOND(8); break;
@@ -1062,11 +1112,14 @@ static void precond_launch(Ctx &c, const double *r, double *z, const int *col_de
   FSD_CUDA(cudaGetLastError());
 }
 
-void launch_precond(Ctx &c, const double *r, double *z) { precond_launch(c, r, z, nullptr, 0, nullptr); }
+// (r is only written for a column past the first, which needs col_dev)
+void launch_precond(Ctx &c, const double *r, double *z) {
+  precond_launch(c, const_cast<double *>(r), z, nullptr, 0, nullptr, nullptr, nullptr);
+}
 
-void launch_precond_col(Ctx &c, const double *V, double *Z, int64_t ld, const int *col_dev,
-                        double *z2) {
-  precond_launch(c, V, Z, col_dev, ld, z2);
+void launch_precond_col(Ctx &c, double *V, double *Z, int64_t ld, const int *col_dev, double *z2,
+                        const double *w, const double *scale_dev) {
+  precond_launch(c, V, Z, col_dev, ld, z2, w, scale_dev);
 }
 
 void launch_rhs(Ctx &c, const double *ft_int, double shear, double *b) {
@@ -1141,8 +1194,8 @@ void launch_nf_pairwise(Ctx &c, uint64_t seed, uint64_t step, double *f) {
   FSD_CUDA(cudaGetLastError());
 }
 
-template void launch_body_rows<float>(Ctx &, const double *, double *, bool);
-template void launch_body_rows<double>(Ctx &, const double *, double *, bool);
+template void launch_body_rows<float>(Ctx &, const double *, double *, bool, const double *);
+template void launch_body_rows<double>(Ctx &, const double *, double *, bool, const double *);
 template void launch_lub_apply<float>(Ctx &, const double *, double *);
 template void launch_lub_apply<double>(Ctx &, const double *, double *);
 

@@ -1075,7 +1075,7 @@ static int realspace_occupancy(size_t smem, int threads) {
 }
 
 template <typename T>
-void launch_realspace(Ctx &c, const double *x, double *y, bool add_constraint, bool) {
+void launch_realspace(Ctx &c, const double *x, double *y, bool add_constraint) {
   ProfScope ps(c, PG_REAL);
   OpData<T> &op = opdata<T>(c);
   const int threads = 256;
@@ -1110,7 +1110,7 @@ void launch_realspace(Ctx &c, const double *x, double *y, bool add_constraint, b
   FSD_CUDA(cudaGetLastError());
 }
 
-template void launch_realspace<float>(Ctx &, const double *, double *, bool, bool);
-template void launch_realspace<double>(Ctx &, const double *, double *, bool, bool);
+template void launch_realspace<float>(Ctx &, const double *, double *, bool);
+template void launch_realspace<double>(Ctx &, const double *, double *, bool);
 
 }  // namespace fsd

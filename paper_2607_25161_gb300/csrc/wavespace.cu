@@ -1057,6 +1057,51 @@ __global__ void __launch_bounds__(256) k_spread_v4(int Nt, const float4 *__restr
   }
 }
 
+// Bead-row components of the read-out from its twelve window sums (u, then the
+// gradient G_ab row by row): component k = sum of up to three coef[k][t] a[idx]
+// plus, in a Lees-Edwards box (d/dy = d/ds_y - tau d/ds_x on the sheared
+// window), tau coef[k][3] a[idx[k][3]].
+__device__ const int kReadIdx[11][4] = {{0, 0, 0, 0}, {1, 1, 1, 1}, {2, 2, 2, 2}, {10, 8, 8, 9}, {5, 9, 9, 9},
+                                        {6, 4, 4, 3}, {3, 7, 7, 6}, {11, 3, 7, 6}, {4, 6, 6, 3}, {5, 9, 9, 9},
+                                        {8, 10, 10, 9}};
+#define FSD_R2I 0.70710678118654752440
+#define FSD_R6I 0.40824829046386301637
+__device__ const double kReadCoef[11][4] = {
+    {1.0, 0.0, 0.0, 0.0}, {1.0, 0.0, 0.0, 0.0}, {1.0, 0.0, 0.0, 0.0},
+    {0.5, -0.5, 0.0, -0.5}, {0.5, -0.5, 0.0, 0.0}, {0.5, -0.5, 0.0, 0.5},
+    {FSD_R2I, -FSD_R2I, 0.0, FSD_R2I}, {2.0 * FSD_R6I, -FSD_R6I, -FSD_R6I, FSD_R6I},
+    {FSD_R2I, FSD_R2I, 0.0, -FSD_R2I}, {FSD_R2I, FSD_R2I, 0.0, 0.0}, {FSD_R2I, FSD_R2I, 0.0, -FSD_R2I}};
+#undef FSD_R2I
+#undef FSD_R6I
+
+// Every lane holds all twelve sums: lane k < 11 writes component k.
+template <typename T>
+__device__ __forceinline__ void read_out(const T *acc, int lane, int i, double *y, double scale, double tau,
+                                         bool set) {
+  if (lane > 11) return;
+  double v = 0.0;
+  if (lane < 11) {
+    const int *ix = kReadIdx[lane];
+    const double *cf = kReadCoef[lane];
+    auto a = [&](int k) {  // acc[k] without indexing the registers
+      T r = acc[0];
+#pragma unroll
+      for (int q = 1; q < 12; ++q) r = k == q ? acc[q] : r;
+      return (double)r;
+    };
+    v = cf[0] * a(ix[0]);
+    if (lane > 2) v = fma(cf[1], a(ix[1]), v);
+    if (lane == 7) v = fma(cf[2], a(ix[2]), v);
+    if (tau != 0.0) v = fma(tau * cf[3], a(ix[3]), v);
+    v *= scale;
+  }
+  double *o = y + (size_t)i * LDB + lane;
+  if (set)
+    *o = v;
+  else if (lane < 11)
+    *o += v;
+}
+
 // One warp per bead: u = h^3 sum W u_M, G_ab = h^3 sum 2 alpha W y_b u_D,a;
 // omega = (1/2) curl, e = sym G projected; added to the bead row of y.
 // PL: the six fields are planar [6][n^3] (from the fused FFT) instead of
@@ -1064,7 +1109,7 @@ __global__ void __launch_bounds__(256) k_spread_v4(int Nt, const float4 *__restr
 template <typename T, bool PL>
 __global__ void __launch_bounds__(256) k_interp(int Nt, const typename V4Of<T>::type *__restrict__ pos,
                                                 const T *__restrict__ grid, double *y, int n, int P,
-                                                T h, T alpha, T cnorm_h3, TauArg ta_) {
+                                                T h, T alpha, T cnorm_h3, TauArg ta_, bool set) {
   const double tau = tau_of(ta_);
   __shared__ T sw[8][3][kMaxP], sy[8][3][kMaxP];
   __shared__ int si[8][3][kMaxP];
@@ -1121,28 +1166,7 @@ __global__ void __launch_bounds__(256) k_interp(int Nt, const typename V4Of<T>::
   for (int off = 16; off > 0; off >>= 1)
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], off);
-  if (lane != 0) return;
-  double a_[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) a_[k] = (double)acc[k] * (double)cnorm_h3;
-  // Lees-Edwards box: d/dy = d/ds_y - tau d/ds_x on the sheared window
-  const double G00 = a_[3], G01 = a_[4] - tau * a_[3], G02 = a_[5], G10 = a_[6],
-               G11 = a_[7] - tau * a_[6], G12 = a_[8], G20 = a_[9], G21 = a_[10] - tau * a_[9],
-               G22 = a_[11];
-  const double r2i = 0.70710678118654752440, r6i = 0.40824829046386301637,
-               s2 = 1.41421356237309504880;
-  double *yr = y + (size_t)i * LDB;
-  yr[0] += a_[0];
-  yr[1] += a_[1];
-  yr[2] += a_[2];
-  yr[3] += 0.5 * (G21 - G12);
-  yr[4] += 0.5 * (G02 - G20);
-  yr[5] += 0.5 * (G10 - G01);
-  yr[6] += r2i * (G00 - G11);
-  yr[7] += r6i * (2.0 * G22 - G00 - G11);
-  yr[8] += s2 * 0.5 * (G01 + G10);
-  yr[9] += s2 * 0.5 * (G02 + G20);
-  yr[10] += s2 * 0.5 * (G12 + G21);
+  read_out(acc, lane, i, y, (double)cnorm_h3, tau, set);
 }
 
 // The sums of k_interp from interleaved fields [n^3][8], factored by grid
@@ -1156,7 +1180,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_interp_rows(int Nt, const typename V4Of<T>::type *__restrict__ pos,
                                                      const T *__restrict__ grid, double *y, int n,
                                                      int P, T h, T alpha, T cnorm_h3, TauArg ta_,
-                                                     FastDiv fp) {
+                                                     FastDiv fp, bool set) {
   const double tau = tau_of(ta_);
   __shared__ T sw[8][3][kMaxP], sy[8][3][kMaxP], swx[8][kMaxP];
   __shared__ int si[8][3][kMaxP];
@@ -1214,46 +1238,8 @@ __global__ void __launch_bounds__(256) k_interp_rows(int Nt, const typename V4Of
   for (int off = 16; off > 0; off >>= 1)
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], off);
-  if (lane != 0) return;
-  double a_[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) a_[k] = (double)acc[k] * (double)cnorm_h3;
-  // Lees-Edwards box: d/dy = d/ds_y - tau d/ds_x on the sheared window
-  const double G00 = a_[3], G01 = a_[4] - tau * a_[3], G02 = a_[5], G10 = a_[6],
-               G11 = a_[7] - tau * a_[6], G12 = a_[8], G20 = a_[9], G21 = a_[10] - tau * a_[9],
-               G22 = a_[11];
-  const double r2i = 0.70710678118654752440, r6i = 0.40824829046386301637,
-               s2 = 1.41421356237309504880;
-  double *yr = y + (size_t)i * LDB;
-  yr[0] += a_[0];
-  yr[1] += a_[1];
-  yr[2] += a_[2];
-  yr[3] += 0.5 * (G21 - G12);
-  yr[4] += 0.5 * (G02 - G20);
-  yr[5] += 0.5 * (G10 - G01);
-  yr[6] += r2i * (G00 - G11);
-  yr[7] += r6i * (2.0 * G22 - G00 - G11);
-  yr[8] += s2 * 0.5 * (G01 + G10);
-  yr[9] += s2 * 0.5 * (G02 + G20);
-  yr[10] += s2 * 0.5 * (G12 + G21);
+  read_out(acc, lane, i, y, (double)cnorm_h3, tau, set);
 }
-
-// Bead-row components of the read-out from its twelve window sums (u, then the
-// gradient G_ab row by row): component k = sum of up to three coef[k][t] a[idx]
-// plus, in a Lees-Edwards box (d/dy = d/ds_y - tau d/ds_x on the sheared
-// window), tau coef[k][3] a[idx[k][3]].
-__device__ const int kReadIdx[11][4] = {{0, 0, 0, 0}, {1, 1, 1, 1}, {2, 2, 2, 2}, {10, 8, 8, 9}, {5, 9, 9, 9},
-                                        {6, 4, 4, 3}, {3, 7, 7, 6}, {11, 3, 7, 6}, {4, 6, 6, 3}, {5, 9, 9, 9},
-                                        {8, 10, 10, 9}};
-#define FSD_R2I 0.70710678118654752440
-#define FSD_R6I 0.40824829046386301637
-__device__ const double kReadCoef[11][4] = {
-    {1.0, 0.0, 0.0, 0.0}, {1.0, 0.0, 0.0, 0.0}, {1.0, 0.0, 0.0, 0.0},
-    {0.5, -0.5, 0.0, -0.5}, {0.5, -0.5, 0.0, 0.0}, {0.5, -0.5, 0.0, 0.5},
-    {FSD_R2I, -FSD_R2I, 0.0, FSD_R2I}, {2.0 * FSD_R6I, -FSD_R6I, -FSD_R6I, FSD_R6I},
-    {FSD_R2I, FSD_R2I, 0.0, -FSD_R2I}, {FSD_R2I, FSD_R2I, 0.0, 0.0}, {FSD_R2I, FSD_R2I, 0.0, -FSD_R2I}};
-#undef FSD_R2I
-#undef FSD_R6I
 
 // FP32 interpolation from bricked fields (grids whose side is a multiple of
 // 4): the sums of k_interp, one warp per bead.  A lane owns one (y, z) row of
@@ -1272,7 +1258,7 @@ __device__ const double kReadCoef[11][4] = {
 __global__ void __launch_bounds__(256, 3) k_interp_brick(int Nt, const float4 *__restrict__ pos,
                                                          const float *__restrict__ field, double *y,
                                                          int n, int P, float h, float alpha,
-                                                         float cnorm_h3, TauArg ta_) {
+                                                         float cnorm_h3, TauArg ta_, bool set) {
   __shared__ float4 zt[8][kMaxP + 2];  // z of the window's bricks: w, w (z - p_z), field offset
   __shared__ float red[8][12];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1370,7 +1356,10 @@ __global__ void __launch_bounds__(256, 3) k_interp_brick(int Nt, const float4 *_
     if (lane == 7) v = fma(cf[2], (double)red[warp][ix[2]], v);
     const double tau = tau_of(ta_);
     if (tau != 0.0) v = fma(tau * cf[3], (double)red[warp][ix[3]], v);
-    y[(size_t)i * LDB + lane] += v * (double)cnorm_h3;
+    double *o = y + (size_t)i * LDB + lane;
+    *o = set ? v * (double)cnorm_h3 : *o + v * (double)cnorm_h3;
+  } else if (set && lane == 11) {
+    y[(size_t)i * LDB + 11] = 0.0;
   }
 }
 
@@ -1750,9 +1739,9 @@ static int fit_log2_lines(int want, int lines_per_unit, int n, int ntw) {
 }
 
 // Inverse y and x transforms of the fields held in spec (after the z pass),
-// then interpolation: y += h^3 sum W (fields) per bead.
+// then interpolation: y += h^3 sum W (fields) per bead, or y = with set.
 template <typename T>
-static void wave_tail(Ctx &c, OpData<T> &op, Cx<T> *spec, double *y) {
+static void wave_tail(Ctx &c, OpData<T> &op, Cx<T> *spec, double *y, bool set) {
   const int n = c.n, P = c.P;
   const T h = (T)c.h, alpha = (T)c.alpha;
   const double cn = std::pow(c.alpha / kPi, 1.5);
@@ -1792,14 +1781,14 @@ static void wave_tail(Ctx &c, OpData<T> &op, Cx<T> *spec, double *y) {
   if (planar && n % 4 == 0)
     k_interp_brick<<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p,
                                                             (const float *)op.gout.p, y, n, P, (float)h,
-                                                            (float)alpha, (float)(cn * h3), tau_arg(c));
+                                                            (float)alpha, (float)(cn * h3), tau_arg(c), set);
   else if (planar)
     k_interp<T, true><<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, posp<T>(c), op.gout.p, y, n, P,
-                                                              h, alpha, (T)(cn * h3), tau_arg(c));
+                                                              h, alpha, (T)(cn * h3), tau_arg(c), set);
   else
     k_interp_rows<T><<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, posp<T>(c), op.gout.p, y, n,
                                                               P, h, alpha, (T)(cn * h3),
-                                                              tau_arg(c), make_fastdiv(P));
+                                                              tau_arg(c), make_fastdiv(P), set);
   FSD_LAUNCHED(c);
   FSD_CUDA(cudaGetLastError());
 }
@@ -1896,7 +1885,7 @@ void refresh_le_tables(Ctx &c) {
 }
 
 template <typename T>
-void launch_wavespace(Ctx &c, const double *x, double *y) {
+void launch_wavespace(Ctx &c, const double *x, double *y, bool set) {
   OpData<T> &op = opd<T>(c);
   const int n = c.n, P = c.P;
   const T h = (T)c.h, alpha = (T)c.alpha;
@@ -1982,11 +1971,11 @@ void launch_wavespace(Ctx &c, const double *x, double *y) {
     FSD_CUDA(cudaGetLastError());
   }
   }
-  wave_tail<T>(c, op, spec, y);
+  wave_tail<T>(c, op, spec, y, set);
 }
 
-template void launch_wavespace<float>(Ctx &, const double *, double *);
-template void launch_wavespace<double>(Ctx &, const double *, double *);
+template void launch_wavespace<float>(Ctx &, const double *, double *, bool);
+template void launch_wavespace<double>(Ctx &, const double *, double *, bool);
 
 template <typename T>
 void launch_brownian_wave(Ctx &c, const double *field, uint64_t seed, uint64_t step, double *out) {
@@ -2034,7 +2023,7 @@ void launch_brownian_wave(Ctx &c, const double *field, uint64_t seed, uint64_t s
     FSD_CUDA(cudaGetLastError());
   }
   FSD_CUDA(cudaMemsetAsync(out, 0, (size_t)c.nunk * sizeof(double), c.stream));
-  wave_tail<T>(c, op, spec, out);
+  wave_tail<T>(c, op, spec, out, false);
 }
 template void launch_brownian_wave<float>(Ctx &, const double *, uint64_t, uint64_t, double *);
 template void launch_brownian_wave<double>(Ctx &, const double *, uint64_t, uint64_t, double *);
@@ -2240,10 +2229,11 @@ extern "C" fsd_status fsd_apply_wave_noalloc(int64_t n_beads, const double *bead
   f->x_inv(st, sp, gout, twc);
   const float cnh3 = (float)(cn * h * h * h);
   if (n % 4 == 0)
-    k_interp_brick<<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3, TauArg());
+    k_interp_brick<<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3, TauArg(),
+                                              true);
   else
     k_interp<float, true><<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3,
-                                                       TauArg());
+                                                       TauArg(), true);
   k_na_stage_out<<<(nb + 127) / 128, 128, 0, st>>>(nb, y, out);
   if (cudaGetLastError() != cudaSuccess) return FSD_ECUDA;
   return FSD_OK;
