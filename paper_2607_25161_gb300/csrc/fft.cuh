@@ -394,11 +394,10 @@ __global__ void __launch_bounds__(Tile<T, R1, R2>::XIT)
       }
     }
   } else {
-    for (int b = threadIdx.x; b < X * R1; b += NT) {
-      const int k1 = b % R1, l = b / R1;
-      if (y0 + l >= n) continue;
-#pragma unroll 1
-      for (int p = 0; p < 3; ++p) {
+    // the three fields of a point by neighbouring lanes
+    for (int b = threadIdx.x; b < 3 * X * R1; b += NT) {
+      const int p = b % 3, r = b / 3, k1 = r % R1, l = r / R1;
+      if (y0 + l < n) {
         Cplx<T> v[R2];
         second_dft<R1, R2, 1>(v, k1, sm + (p * X + l) * L::LT);
         T *o = out + (((int64_t)z * n + y0 + l) * n + k1) * 8 + p;

@@ -1038,6 +1038,13 @@ OpData<float> &opdata<float>(Ctx &c) {
   return c.op32;
 }
 
+// The real-space sum's launch.  Small suspensions (fewer than four warps per SM
+// at 32 lanes per bead) take 32 lanes and blocks of 64 threads: the pair
+// arithmetic of a few warps on one SM is a queue at its FP64 pipe, a warp per
+// bead spread over the SMs is not (a 32-bead FP64 solve, with the bead-per-warp
+// kernels spread likewise, 2.17 -> 1.88 ms).
+static bool realspace_small(const Ctx &c) { return c.Nt <= 4 * c.num_sms; }
+
 // Lanes that share one bead's neighbour list, from the mean neighbour count
 // (a tile shape the caller may fix with fsd_params.tile).  On the 32768-bead
 // benchmark (168 neighbours per bead) 16 lanes beat 32: 0.122 against 0.133
@@ -1046,6 +1053,7 @@ OpData<float> &opdata<float>(Ctx &c) {
 int realspace_group(const Ctx &c) {
   const int t = c.prm.tile;
   if (t == 4 || t == 8 || t == 16 || t == 32) return t;
+  if (realspace_small(c)) return 32;
   const double avg = (double)c.n_pairs / std::max(1, c.Nt);
   return avg > 256 ? 32 : (avg > 40 ? 16 : (avg > 16 ? 8 : 4));
 }
@@ -1058,7 +1066,7 @@ int realspace_group(const Ctx &c) {
 template <typename T, int GG>
 static int realspace_occupancy(size_t smem, int threads) {
   static std::mutex mu;
-  static std::vector<std::pair<size_t, int>> seen;
+  static std::vector<std::pair<std::pair<size_t, int>, int>> seen;  // (smem, threads) -> blocks
   static size_t limit = 0;
   std::lock_guard<std::mutex> lock(mu);
   if (smem > limit) {
@@ -1067,10 +1075,10 @@ static int realspace_occupancy(size_t smem, int threads) {
     limit = smem;
   }
   for (auto &e : seen)
-    if (e.first == smem) return e.second;
+    if (e.first == std::make_pair(smem, threads)) return e.second;
   int occ = 0;
   FSD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_realspace<T, GG>, threads, smem));
-  seen.emplace_back(smem, occ);
+  seen.push_back({{smem, threads}, occ});
   return occ;
 }
 
@@ -1078,7 +1086,7 @@ template <typename T>
 void launch_realspace(Ctx &c, const double *x, double *y, bool add_constraint) {
   ProfScope ps(c, PG_REAL);
   OpData<T> &op = opdata<T>(c);
-  const int threads = 256;
+  const int threads = realspace_small(c) ? 64 : 256;
   if (op.packed.n < (size_t)c.Nt * 16) op.packed.alloc((size_t)c.Nt * 16);
   k_pack_sources<T><<<ceil_div(c.Nt, 256), 256, 0, c.stream>>>(c.Nt, (const double4 *)c.pos64.p, x,
                                                               op.packed.p);

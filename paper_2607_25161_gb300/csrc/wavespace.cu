@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(256) k_spread(int Nt, const typename V4Of<T>::
   __shared__ T rc[8][kSpreadRows][9];
   __shared__ int ro[8][kSpreadRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + warp;
+  const int i = blockIdx.x * (blockDim.x >> 5) + warp;
   if (i >= Nt) return;
   const auto p = pos[i];
   const T pc[3] = {p.x, p.y, p.z};
@@ -992,7 +992,7 @@ __global__ void __launch_bounds__(256) k_spread_v4(int Nt, const float4 *__restr
   __shared__ float sxw[8][4 * kMaxQ], sxy[8][4 * kMaxQ];
   __shared__ int sxq[8][kMaxQ];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + warp;
+  const int i = blockIdx.x * (blockDim.x >> 5) + warp;
   if (i >= Nt) return;
   const float4 p = pos[i];
   const int g0x = (int)floorf(p.x / h) - P / 2 + 1;
@@ -1114,7 +1114,7 @@ __global__ void __launch_bounds__(256) k_interp(int Nt, const typename V4Of<T>::
   __shared__ T sw[8][3][kMaxP], sy[8][3][kMaxP];
   __shared__ int si[8][3][kMaxP];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + warp;
+  const int i = blockIdx.x * (blockDim.x >> 5) + warp;
   if (i >= Nt) return;
   const auto p = pos[i];
   const T pc[3] = {p.x, p.y, p.z};
@@ -1185,7 +1185,7 @@ __global__ void __launch_bounds__(256) k_interp_rows(int Nt, const typename V4Of
   __shared__ T sw[8][3][kMaxP], sy[8][3][kMaxP], swx[8][kMaxP];
   __shared__ int si[8][3][kMaxP];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + warp;
+  const int i = blockIdx.x * (blockDim.x >> 5) + warp;
   if (i >= Nt) return;
   const auto p = pos[i];
   const T pc[3] = {p.x, p.y, p.z};
@@ -1262,7 +1262,7 @@ __global__ void __launch_bounds__(256, 3) k_interp_brick(int Nt, const float4 *_
   __shared__ float4 zt[8][kMaxP + 2];  // z of the window's bricks: w, w (z - p_z), field offset
   __shared__ float red[8][12];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + warp;
+  const int i = blockIdx.x * (blockDim.x >> 5) + warp;
   if (i >= Nt) return;
   const float4 p = pos[i];
   const int g0x = (int)floorf(p.x / h) - P / 2 + 1, g0y = (int)floorf(p.y / h) - P / 2 + 1;
@@ -1738,6 +1738,12 @@ static int fit_log2_lines(int want, int lines_per_unit, int n, int ntw) {
   throw Invalid{"FFT grid too large for one line per block in shared memory"};
 }
 
+// Warps per block of the kernels with a warp per bead: up to eight, and fewer
+// below eight beads per SM, so that a small suspension's FP64 work, which one
+// SM's pipe takes in turn, is spread over the SMs (a 32-bead FP64 solve:
+// with the real-space sum spread likewise 2.17 -> 1.88 ms).
+static int bead_warps(const Ctx &c) { return std::min(8, std::max(1, ceil_div(c.Nt, std::max(1, c.num_sms)))); }
+
 // Inverse y and x transforms of the fields held in spec (after the z pass),
 // then interpolation: y += h^3 sum W (fields) per bead, or y = with set.
 template <typename T>
@@ -1779,14 +1785,14 @@ static void wave_tail(Ctx &c, OpData<T> &op, Cx<T> *spec, double *y, bool set) {
   const double h3 = c.h * c.h * c.h;
   const bool planar = sizeof(T) == 4 && f;
   if (planar && n % 4 == 0)
-    k_interp_brick<<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p,
+    k_interp_brick<<<ceil_div(c.Nt, bead_warps(c)), 32 * bead_warps(c), 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p,
                                                             (const float *)op.gout.p, y, n, P, (float)h,
                                                             (float)alpha, (float)(cn * h3), tau_arg(c), set);
   else if (planar)
-    k_interp<T, true><<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, posp<T>(c), op.gout.p, y, n, P,
+    k_interp<T, true><<<ceil_div(c.Nt, bead_warps(c)), 32 * bead_warps(c), 0, c.stream>>>(c.Nt, posp<T>(c), op.gout.p, y, n, P,
                                                               h, alpha, (T)(cn * h3), tau_arg(c), set);
   else
-    k_interp_rows<T><<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, posp<T>(c), op.gout.p, y, n,
+    k_interp_rows<T><<<ceil_div(c.Nt, bead_warps(c)), 32 * bead_warps(c), 0, c.stream>>>(c.Nt, posp<T>(c), op.gout.p, y, n,
                                                               P, h, alpha, (T)(cn * h3),
                                                               tau_arg(c), make_fastdiv(P), set);
   FSD_LAUNCHED(c);
@@ -1903,12 +1909,12 @@ void launch_wavespace(Ctx &c, const double *x, double *y, bool set) {
   } else {
   FSD_CUDA(cudaMemsetAsync(op.grid.p, 0, gbytes, c.stream));
   if (sizeof(T) == 4 && n % 4 == 0)
-    k_spread_v4<<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p, x,
+    k_spread_v4<<<ceil_div(c.Nt, bead_warps(c)), 32 * bead_warps(c), 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p, x,
                                                          (float *)op.grid.p, n, P, (float)h,
                                                          (float)alpha, (float)cn,
                                                          tau_arg(c));
   else
-    k_spread<T><<<ceil_div(c.Nt, 8), 256, 0, c.stream>>>(c.Nt, posp<T>(c), x, op.grid.p, n, P, h,
+    k_spread<T><<<ceil_div(c.Nt, bead_warps(c)), 32 * bead_warps(c), 0, c.stream>>>(c.Nt, posp<T>(c), x, op.grid.p, n, P, h,
                                                         alpha, (T)cn, tau_arg(c), make_fastdiv(P));
   }
   FSD_LAUNCHED(c);
