@@ -617,8 +617,7 @@ static void setup_impl(Ctx &c, int64_t n_beads, const double *bead_pos, const in
   c.flags.alloc(kFlags);
   FSD_CUDA(cudaMallocHost(&c.h_flags, kFlags * sizeof(int)));
   c.brow.alloc(Nt + 1);
-  c.op64.bdiag.alloc((size_t)Nt * 36);
-  c.op32.bdiag.alloc((size_t)Nt * 36);
+  if (p.nf_sampler == FSD_NF_LANCZOS) c.bdiag.alloc((size_t)Nt * 36);
   c.pdiag.alloc((size_t)Nt * 36);
   c.schur.alloc((size_t)N * 36);
   c.piv.alloc((size_t)N * 6);

@@ -373,7 +373,7 @@ void brownian_sample(Ctx &c, double kT, double dt, uint64_t seed, uint64_t step,
     // blocks are (nearly) the identity
     if (c.bgain.n < (size_t)c.Nt * 72) c.bgain.alloc((size_t)c.Nt * 72);
     double *Lb = c.bgain.p, *G = c.bgain.p + (size_t)c.Nt * 36;
-    k_block_chol<<<ceil_div(c.Nt, 64), 64, 0, c.stream>>>(c.Nt, c.op64.bdiag.p, Lb, G);
+    k_block_chol<<<ceil_div(c.Nt, 64), 64, 0, c.stream>>>(c.Nt, c.bdiag.p, Lb, G);
     FSD_LAUNCHED(c);
     if (c.bwork2.n < (size_t)n) c.bwork2.alloc(n);
     double *tmp = c.bwork2.p;
@@ -381,8 +381,8 @@ void brownian_sample(Ctx &c, double kT, double dt, uint64_t seed, uint64_t step,
     auto nf_op = [&](const double *x, double *y) {
       k_block_apply<<<ceil_div(c.Nt, 128), 128, 0, c.stream>>>(c.Nt, G, 1, x, tmp);
       FSD_LAUNCHED(c);
-      k_bsr_bead<<<ceil_div(c.Nt, 128), 128, 0, c.stream>>>(c.Nt, c.brow.p, c.bcol.p, c.op64.bval.p,
-                                                            c.op64.bdiag.p, tmp, y);
+      k_bsr_bead<<<ceil_div(c.Nt, 128), 128, 0, c.stream>>>(c.Nt, c.brow.p, c.bcol.p, c.bval.p,
+                                                            c.bdiag.p, tmp, y);
       FSD_LAUNCHED(c);
       k_block_apply<<<ceil_div(c.Nt, 128), 128, 0, c.stream>>>(c.Nt, G, 0, y, y);
       FSD_LAUNCHED(c);

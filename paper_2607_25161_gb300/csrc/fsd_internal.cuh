@@ -85,8 +85,6 @@ struct OpData {
   DBuf<T> gout;       // velocity fields for interpolation, interleaved: [n^3][8] (6 used)
   DBuf<T> green;      // [m = kx^2+ky^2+kz^2][3]: (A fM^2, A fM fD, A fD^2)
   DBuf<T> twiddle;    // [n] complex: exp(-2 pi i t / n)
-  DBuf<T> bval;       // lubrication BSR off-diagonal blocks [nnz][36]
-  DBuf<T> bdiag;      // lubrication BSR diagonal blocks [Nt][36]
   DBuf<T> pos;        // wrapped positions [Nt][4] (x, y, z, 0)
   DBuf<T> lever;      // r_b = x_b - X_J [Nt][4]
   DBuf<T> packed;     // per bead (x, y, z, F, L, S6, 0) in the operator precision [Nt][16]
@@ -203,7 +201,9 @@ struct Ctx {
   int *h_flags = nullptr;  // pinned
   // ---- lubrication BSR (rows = beads; diagonal separate)
   DBuf<int> brow, bcol;
-  DBuf<double> lpair;  // per directed pair (n, r, A, B, D, within r_p) [nnz][8]
+  DBuf<double> lpair;   // per directed pair (n, r, A, B, D, within r_p) [nnz][8]
+  DBuf<float> lpair32;  // the same in FP32 (n, r/2, A, B, D, 0) [nnz][8]
+  DBuf<double> bval, bdiag;  // 6x6 blocks [nnz][36], [Nt][36] (FSD_NF_LANCZOS only)
   int nnz_cap = 0;
   // ---- preconditioner
   DBuf<double> schur;  // [N][36] LU factors

@@ -45,7 +45,7 @@ struct GState {
 struct GraphKey {
   int mixed, warm, has_ft, integrate, with_str, group, lub, brown, add_vel, str_hydro, le;
   double shear, dt, brown_scale, tilt;
-  const void *nbr, *lnbr, *bcol, *bval64, *bval32, *lpair, *packed64, *packed32;
+  const void *nbr, *lnbr, *bcol, *lpair, *lpair32, *packed64, *packed32;
   int cap, lcap;
   int64_t nunk;
   bool operator==(const GraphKey &o) const { return std::memcmp(this, &o, sizeof(*this)) == 0; }
@@ -593,9 +593,8 @@ static GraphKey make_key(Ctx &c, const GraphRun &o) {
   k.nbr = c.nbr.p;
   k.lnbr = c.lnbr.p;
   k.bcol = c.bcol.p;
-  k.bval64 = c.op64.bval.p;
-  k.bval32 = c.op32.bval.p;
   k.lpair = c.lpair.p;
+  k.lpair32 = c.lpair32.p;
   k.packed64 = c.op64.packed.p;
   k.packed32 = c.op32.packed.p;
   k.cap = c.cap;

@@ -118,9 +118,10 @@ __device__ __forceinline__ void min_image(double &d0, double &d1, double &d2, do
   le_image(d0, d1, d2, L, tilt);
 }
 
-// Thread per directed pair: its record, and its off-diagonal block in CSR
-// order, staged in shared memory so that the 36 values of a block are stored
-// by neighbouring lanes.  The row is found by bisection in the row starts.
+// Thread per directed pair: its record in both precisions and, for the Lanczos
+// sampler of the near-field forces (bval64 non-null), its off-diagonal block in
+// CSR order, staged in shared memory so that the 36 values of a block are
+// stored by neighbouring lanes.  The row is found by bisection in the row starts.
 // Bound by FP64 arithmetic (a logarithm, a square root and the divisions).
 // A thread per bead walked its pairs one after the other, a dependent FP64
 // chain with a third of the lanes idle, and wrote 288-byte strides: with the
@@ -128,7 +129,7 @@ __device__ __forceinline__ void min_image(double &d0, double &d1, double &d2, do
 constexpr int kLP = 64;  // pairs per block
 __global__ void __launch_bounds__(kLP) k_lub_pairs(
     int Nt, int nnz, const double4 *__restrict__ pos, const int *__restrict__ lnbr, int lcap,
-    const int *__restrict__ brow, int *bcol, PairRec *rec, double *bval64, float *bval32, double L,
+    const int *__restrict__ brow, int *bcol, PairRec *rec, float4 *rec32, double *bval64, double L,
     double tilt, double a, double eta, double rcut, double rp, LubModel lm) {
   __shared__ double sb[kLP][37];
   const int s0 = blockIdx.x * kLP, s = s0 + threadIdx.x;
@@ -157,25 +158,26 @@ __global__ void __launch_bounds__(kLP) k_lub_pairs(
     p.pre = p.r < rp ? 1.0 : 0.0;
     bcol[s] = j;
     rec[s] = p;
-    double R[36];
-    pair_block_ij(p, R);
+    rec32[2 * (size_t)s] = make_float4((float)p.n[0], (float)p.n[1], (float)p.n[2], (float)(0.5 * p.r));
+    rec32[2 * (size_t)s + 1] = make_float4((float)p.A, (float)p.B, (float)p.D, 0.f);
+    if (bval64) {
+      double R[36];
+      pair_block_ij(p, R);
 #pragma unroll
-    for (int e = 0; e < 36; ++e) sb[threadIdx.x][e] = R[e];
+      for (int e = 0; e < 36; ++e) sb[threadIdx.x][e] = R[e];
+    }
   }
+  if (!bval64) return;
   __syncthreads();
   const int m = min(kLP, nnz - s0) * 36;
-  for (int e = threadIdx.x; e < m; e += kLP) {
-    const double v = sb[e / 36][e % 36];
-    bval64[(size_t)s0 * 36 + e] = v;
-    bval32[(size_t)s0 * 36 + e] = (float)v;
-  }
+  for (int e = threadIdx.x; e < m; e += kLP) bval64[(size_t)s0 * 36 + e] = sb[e / 36][e % 36];
 }
 
-// Thread per bead: the diagonal block and the preconditioner's (pairs closer
-// than r_p only) from the pair records; R_ii has 15 distinct entries.
+// Thread per bead: the diagonal block (for the Lanczos sampler: bdiag64 non-null)
+// and the preconditioner's (pairs closer than r_p only) from the pair records; R_ii has 15 distinct entries.
 __global__ void __launch_bounds__(kLP) k_lub_diag(int Nt, const int *__restrict__ brow,
                                                   const PairRec *__restrict__ rec, double *bdiag64,
-                                                  float *bdiag32, double *pdiag) {
+                                                  double *pdiag) {
   __shared__ double sb[kLP][37];
   const int i0 = blockIdx.x * kLP, i = i0 + threadIdx.x;
   double acc[2][15];
@@ -204,6 +206,7 @@ __global__ void __launch_bounds__(kLP) k_lub_diag(int Nt, const int *__restrict_
   const int m = min(kLP, Nt - i0) * 36;
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
+    if (q == 0 && !bdiag64) continue;
     const double *v = acc[q];
     const double G[9] = {v[0], v[3], v[4], v[3], v[1], v[5], v[4], v[5], v[2]};
     const double N[9] = {0, -v[8], v[7], v[8], 0, -v[6], -v[7], v[6], 0};
@@ -222,12 +225,7 @@ __global__ void __launch_bounds__(kLP) k_lub_diag(int Nt, const int *__restrict_
     __syncthreads();
     for (int e = threadIdx.x; e < m; e += kLP) {
       const double w = sb[e / 36][e % 36];
-      if (q == 0) {
-        bdiag64[(size_t)i0 * 36 + e] = w;
-        bdiag32[(size_t)i0 * 36 + e] = (float)w;
-      } else {
-        pdiag[(size_t)i0 * 36 + e] = w;
-      }
+      (q == 0 ? bdiag64 : pdiag)[(size_t)i0 * 36 + e] = w;
     }
   }
 }
@@ -475,16 +473,35 @@ struct LV<float> {
   using type = float4;
 };
 
+// The pair's record in the operator precision: n, r/2, A, B, D.
+template <typename T>
+struct RowRec {
+  T n0, n1, n2, hr, A, B, D;
+};
+__device__ __forceinline__ RowRec<double> row_rec(const PairRec *rec, const float *, int k, double) {
+  const PairRec p = rec[k];
+  return {p.n[0], p.n[1], p.n[2], 0.5 * p.r, p.A, p.B, p.D};
+}
+__device__ __forceinline__ RowRec<float> row_rec(const PairRec *, const float *rec32, int k, float) {
+  const float4 a = __ldg((const float4 *)rec32 + 2 * (size_t)k), b = __ldg((const float4 *)rec32 + 2 * (size_t)k + 1);
+  return {a.x, a.y, a.z, a.w, b.x, b.y, b.z};
+}
+
 // LPA lanes per aggregate (a power of two covering its beads): y2_J =
-// Sigma B^T x1 - [Sigma R Sigma^T x2]_J, the BSR row of every bead evaluated
-// with its neighbours' rigid velocities formed on the fly from x2 (constraint
-// scatter fused into the SpMV).
+// Sigma B^T x1 - [Sigma R Sigma^T x2]_J, a bead per lane, its pairs' forces
+// formed from the relative motion of the two surfaces (the pair model's own
+// form: the common motion cancels before it is multiplied by the resistance)
+// with the neighbours' rigid velocities formed on the fly from x2.  Bound by the
+// loads: a pair's record is 32 bytes in FP32, where its 6x6 block was 144, read
+// by 36 scalar loads that touched a line per lane (with the beads' diagonal
+// blocks 21 us per FP32 application on 32768 beads, now 14; FP64 on 4096 beads
+// 41 -> 36 us).
 template <typename T, int LPA>
 __global__ void __launch_bounds__(256) k_body_rows(
     int N, const int *__restrict__ body_start, const int *__restrict__ bead_body,
     const typename LV<T>::type *__restrict__ lever, const double *__restrict__ x, double *y,
-    const int *__restrict__ brow, const int *__restrict__ bcol, const T *__restrict__ bval,
-    const T *__restrict__ bdiag, int with_lub, int64_t off, T sgn_bead, T sgn_lub,
+    const int *__restrict__ brow, const int *__restrict__ bcol, const PairRec *__restrict__ rec,
+    const float *__restrict__ rec32, int with_lub, int64_t off, T sgn_bead, T sgn_lub,
     const double *__restrict__ add) {
   // the blocks past the aggregates': bead rows += add (the wave-space part of an
   // overlapped application), 256 threads x 2 pairs each
@@ -525,35 +542,29 @@ __global__ void __launch_bounds__(256) k_body_rows(
         v[4] = w1;
         v[5] = w2;
       }
-      T g[6];
-      const T *D = bdiag + (size_t)b * 36;
-#pragma unroll
-      for (int a = 0; a < 6; ++a) {
-        T s = T(0);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) s += D[6 * a + c] * v[c];
-        g[a] = s;
-      }
-      for (int k = brow[b]; k < brow[b + 1]; ++k) {
+      T g[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};  // R v of this bead
+      const int ke = brow[b + 1];
+      for (int k = brow[b]; k < ke; ++k) {
         const int cidx = bcol[k];
+        const RowRec<T> p = row_rec(rec, rec32, k, T(0));
         const double *u = x + off + 6 * (size_t)bead_body[cidx];
         const auto rc = lever[cidx];
         const T u0 = (T)u[0], u1 = (T)u[1], u2 = (T)u[2], w0 = (T)u[3], w1 = (T)u[4], w2 = (T)u[5];
-        T vc[6];
-        vc[0] = u0 + w1 * rc.z - w2 * rc.y;
-        vc[1] = u1 + w2 * rc.x - w0 * rc.z;
-        vc[2] = u2 + w0 * rc.y - w1 * rc.x;
-        vc[3] = w0;
-        vc[4] = w1;
-        vc[5] = w2;
-        const T *Bk = bval + (size_t)k * 36;
-#pragma unroll
-        for (int a = 0; a < 6; ++a) {
-          T s = T(0);
-#pragma unroll
-          for (int c = 0; c < 6; ++c) s += Bk[6 * a + c] * vc[c];
-          g[a] += s;
-        }
+        // relative surface velocity and rotation
+        const T h0 = p.hr * (w0 + v[3]), h1 = p.hr * (w1 + v[4]), h2 = p.hr * (w2 + v[5]);
+        const T s0 = u0 + w1 * rc.z - w2 * rc.y - v[0] + p.n1 * h2 - p.n2 * h1;
+        const T s1 = u1 + w2 * rc.x - w0 * rc.z - v[1] + p.n2 * h0 - p.n0 * h2;
+        const T s2 = u2 + w0 * rc.y - w1 * rc.x - v[2] + p.n0 * h1 - p.n1 * h0;
+        const T t0 = v[3] - w0, t1 = v[4] - w1, t2 = v[5] - w2;
+        const T ns = (p.A - p.B) * (p.n0 * s0 + p.n1 * s1 + p.n2 * s2);
+        const T nt = p.n0 * t0 + p.n1 * t1 + p.n2 * t2;
+        const T G0 = p.B * s0 + ns * p.n0, G1 = p.B * s1 + ns * p.n1, G2 = p.B * s2 + ns * p.n2;
+        g[0] -= G0;
+        g[1] -= G1;
+        g[2] -= G2;
+        g[3] += p.D * (t0 - nt * p.n0) - p.hr * (p.n1 * G2 - p.n2 * G1);
+        g[4] += p.D * (t1 - nt * p.n1) - p.hr * (p.n2 * G0 - p.n0 * G2);
+        g[5] += p.D * (t2 - nt * p.n2) - p.hr * (p.n0 * G1 - p.n1 * G0);
       }
 #pragma unroll
       for (int a = 0; a < 6; ++a) f[a] = sgn_bead * f[a] + sgn_lub * g[a];
@@ -997,12 +1008,13 @@ void build_lubrication(Ctx &c) {
   // CSR rows from the lubrication neighbour counts (their total is known from
   // the search)
   const int nnz = (int)c.n_lub;
+  const bool lanczos = c.prm.nf_sampler == FSD_NF_LANCZOS;  // the only user of the 6x6 blocks
   if (nnz > c.nnz_cap || !c.bcol.p) {
     c.nnz_cap = std::max(nnz + nnz / 4 + 64, 64);
     c.bcol.alloc(c.nnz_cap);
-    c.op64.bval.alloc((size_t)c.nnz_cap * 36);
-    c.op32.bval.alloc((size_t)c.nnz_cap * 36);
+    if (lanczos) c.bval.alloc((size_t)c.nnz_cap * 36);
     c.lpair.alloc((size_t)c.nnz_cap * 8);
+    c.lpair32.alloc((size_t)c.nnz_cap * 8);
   }
   k_exclusive_scan<<<1, 1024, 0, c.stream>>>(Nt, c.lcnt.p, c.brow.p, nullptr);
   FSD_LAUNCHED(c);
@@ -1010,11 +1022,11 @@ void build_lubrication(Ctx &c) {
   PairRec *rec = (PairRec *)c.lpair.p;
   if (nnz > 0) {
     k_lub_pairs<<<ceil_div(nnz, kLP), kLP, 0, c.stream>>>(
-        Nt, nnz, (const double4 *)c.pos64.p, c.lnbr.p, c.lcap, c.brow.p, c.bcol.p, rec, c.op64.bval.p,
-        c.op32.bval.p, c.L, c.tilt, c.a, c.eta, rl, c.prm.precond_cutoff, lub_model(c));
+        Nt, nnz, (const double4 *)c.pos64.p, c.lnbr.p, c.lcap, c.brow.p, c.bcol.p, rec,
+        (float4 *)c.lpair32.p, lanczos ? c.bval.p : nullptr, c.L, c.tilt, c.a, c.eta, rl, c.prm.precond_cutoff, lub_model(c));
     FSD_LAUNCHED(c);
   }
-  k_lub_diag<<<ceil_div(Nt, kLP), kLP, 0, c.stream>>>(Nt, c.brow.p, rec, c.op64.bdiag.p, c.op32.bdiag.p,
+  k_lub_diag<<<ceil_div(Nt, kLP), kLP, 0, c.stream>>>(Nt, c.brow.p, rec, lanczos ? c.bdiag.p : nullptr,
                                                      c.pdiag.p);
   FSD_LAUNCHED(c);
   FSD_CUDA(cudaGetLastError());
@@ -1058,13 +1070,12 @@ OpData<float> &opx<float>(Ctx &c) {
 template <typename T>
 static void body_rows_launch(Ctx &c, const double *x, double *y, int lub, T sgn_bead, T sgn_lub,
                              const double *add = nullptr) {
-  OpData<T> &op = opx<T>(c);
   const int64_t off = (int64_t)LDB * c.Nt;
   const int extra = add ? ceil_div(off / 2, 512) : 0;
 #define FSD_BODY_ROWS(LPA)                                                                      \
   k_body_rows<T, LPA><<<ceil_div((int64_t)c.N * LPA, 256) + extra, 256, 0, c.stream>>>(        \
-      c.N, c.body_start.p, c.bead_body.p, lever_ptr<T>(c), x, y, c.brow.p, c.bcol.p, op.bval.p, \
-      op.bdiag.p, lub, off, sgn_bead, sgn_lub, add)
+      c.N, c.body_start.p, c.bead_body.p, lever_ptr<T>(c), x, y, c.brow.p, c.bcol.p, \
+      (const PairRec *)c.lpair.p, c.lpair32.p, lub, off, sgn_bead, sgn_lub, add)
   switch (c.body_lanes) {
     case 4: FSD_BODY_ROWS(4); break;
     case 8: FSD_BODY_ROWS(8); break;
