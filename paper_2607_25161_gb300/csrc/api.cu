@@ -660,13 +660,16 @@ static void setup_impl(Ctx &c, int64_t n_beads, const double *bead_pos, const in
 }
 
 // Geometry-dependent preparation of one solve: positions, neighbour lists,
-// lubrication blocks, Schur LUs (Alg. 1 step 1).
-static void prepare(Ctx &c) {
+// lubrication blocks, Schur LUs (Alg. 1 step 1), and the FP32 spreading's tile
+// lists where the solve applies the FP32 operator (another FP32 application
+// builds them itself).  A mobility application takes the lists alone: the
+// lubrication kernels and, in FP64, the tiles were 0.15 ms of a 1.6 ms call.
+static void prepare(Ctx &c, bool lubrication = true) {
   c.last_warning = FSD_OK;
   launch_wrap_positions(c);
   build_neighbors(c);
-  build_lubrication(c);
-  if (c.spread_gather && !c.tiles_valid) build_spread_tiles(c);
+  if (lubrication) build_lubrication(c);
+  if (c.spread_gather && !c.tiles_valid && c.prm.precision == FSD_MIXED) build_spread_tiles(c);
 }
 
 static void fill_stats(Ctx &c, fsd_stats *st, const KStats &k, double rel, double ms) {
@@ -1319,7 +1322,7 @@ fsd_status fsd_apply_mobility(fsd_ctx *ctx, const double *in, double *out, int p
   if (!ctx || !in || !out || part < 1 || part > 3) return FSD_EINVAL;
   FSD_API_TRY
   Ctx &c = ctx->c;
-  prepare(c);
+  prepare(c, false);
   vec_in(c, in, c.t1.p, true, false);
   double *y = c.t2.p;
   FSD_CUDA(cudaMemsetAsync(y, 0, c.nunk * sizeof(double), c.stream));
