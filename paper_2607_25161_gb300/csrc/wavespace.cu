@@ -1380,6 +1380,16 @@ __device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  F2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ F2 f2_pair(float a, float b) {
+  F2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
 __device__ __forceinline__ F2 f2_both(float v) {
   F2 d;
   asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));
@@ -1435,6 +1445,7 @@ __global__ void k_tile_bin(int Nt, const float4 *__restrict__ pos, float h, int 
 // 72 multiply-adds of a (bead, row) are taken two x points at a time in one
 // instruction (same rounding), 0.152 -> 0.130 ms per application on 32768
 // beads at n = 144, with 10 blocks per SM (12 spill, 0.152; 8: 0.140).
+template <bool LIN>
 __global__ void __launch_bounds__(64, 10) k_spread_gather(int n, int nt, int P, float h, float alpha,
                                                       float cnorm, TauArg ta_,
                                                       const float4 *__restrict__ pos,
@@ -1445,7 +1456,8 @@ __global__ void __launch_bounds__(64, 10) k_spread_gather(int n, int nt, int P, 
   const float tau = (float)tau_of(ta_);
   // records padded to an odd number of 16-byte units (bank spread when the
   // lanes of a warp read different beads)
-  __shared__ __align__(16) float swx[kTCH][20];      // w[8], w * offset[8], pad
+  constexpr int kWX = LIN ? 12 : 20;
+  __shared__ __align__(16) float swx[kTCH][kWX];     // w[8], then the first offset or w * offset[8], pad
   __shared__ __align__(16) float2 syz[kTCH][2][9];   // (w, offset) of y[8] and z[8], pad
   __shared__ __align__(16) float sm[kTCH][12];
   __shared__ unsigned scov[2][kTCH];  // y and z rows of the tile each bead's window reaches
@@ -1490,12 +1502,19 @@ __global__ void __launch_bounds__(64, 10) k_spread_gather(int n, int nt, int P, 
         cov |= (w != 0.f ? 1u : 0u) << k;
         if (d == 0) {
           swx[bi][k] = w;
-          swx[bi][kTS + k] = w * yv;
+          if (!LIN) swx[bi][kTS + k] = w * yv;
         } else {
           syz[bi][d - 1][k] = make_float2(w, yv);
         }
       }
-      if (d > 0) scov[d - 1][bi] = cov;
+      if (d > 0)
+        scov[d - 1][bi] = cov;
+      else if (LIN) {  // offset of the tile's first point from the bead's nearest image
+        int off = gb - g0;
+        if (off < -kTS) off += n;
+        if (off >= P) off -= n;
+        swx[bi][kTS] = float(g0 + off) * h - pc;
+      }
     }
     // moments: F and the dipole D (= S + antisym(L); column 0 takes -tau
     // column 1 in a Lees-Edwards box), with the window norm and 2 alpha
@@ -1557,17 +1576,31 @@ __global__ void __launch_bounds__(64, 10) k_spread_gather(int n, int nt, int P, 
       const float c0 = (m1.x * yy + m1.y * yz) * wyz, c1 = (m1.w * yy + m2.x * yz) * wyz,
                   c2 = (m2.z * yy + m2.w * yz) * wyz;
       const ulonglong2 wa = *(const ulonglong2 *)&swx[bi][0], wb = *(const ulonglong2 *)&swx[bi][4];
-      const ulonglong2 pa = *(const ulonglong2 *)&swx[bi][8], pb = *(const ulonglong2 *)&swx[bi][12];
-      const F2 wx[kTS / 2] = {wa.x, wa.y, wb.x, wb.y}, px[kTS / 2] = {pa.x, pa.y, pb.x, pb.y};
+      const F2 wx[kTS / 2] = {wa.x, wa.y, wb.x, wb.y};
       const F2 g[9] = {f2_both(f0), f2_both(f1), f2_both(f2), f2_both(a0), f2_both(a1),
                        f2_both(a2), f2_both(c0), f2_both(c1), f2_both(c2)};
+      if constexpr (LIN) {
+        const F2 d0 = f2_both(swx[bi][kTS]);
 #pragma unroll
-      for (int k = 0; k < kTS / 2; ++k)
+        for (int k = 0; k < kTS / 2; ++k) {
+          const F2 d = f2_add(d0, f2_pair(float(2 * k) * h, float(2 * k + 1) * h));
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          acc[c][k] = f2_fma(g[c], wx[k], acc[c][k]);
-          acc[3 + c][k] = f2_fma(g[3 + c], px[k], f2_fma(g[6 + c], wx[k], acc[3 + c][k]));
+          for (int c = 0; c < 3; ++c) {
+            acc[c][k] = f2_fma(g[c], wx[k], acc[c][k]);
+            acc[3 + c][k] = f2_fma(f2_fma(g[3 + c], d, g[6 + c]), wx[k], acc[3 + c][k]);
+          }
         }
+      } else {
+        const ulonglong2 pa = *(const ulonglong2 *)&swx[bi][8], pb = *(const ulonglong2 *)&swx[bi][12];
+        const F2 px[kTS / 2] = {pa.x, pa.y, pb.x, pb.y};
+#pragma unroll
+        for (int k = 0; k < kTS / 2; ++k)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            acc[c][k] = f2_fma(g[c], wx[k], acc[c][k]);
+            acc[3 + c][k] = f2_fma(g[3 + c], px[k], f2_fma(g[6 + c], wx[k], acc[3 + c][k]));
+          }
+      }
     }
   }
   const int yg = y0 + iy, zg = z0 + iz;
@@ -1902,10 +1935,11 @@ void launch_wavespace(Ctx &c, const double *x, double *y, bool set) {
   if (sizeof(T) == 4 && c.spread_gather) {
     if (!c.tiles_valid) build_spread_tiles(c);
     const int nt = c.tile_n;
-    k_spread_gather<<<nt * nt * nt, 64, 0, c.stream>>>(n, nt, P, (float)h, (float)alpha, (float)cn,
-                                                       tau_arg(c), (const float4 *)c.wpos32.p,
-                                                       x, c.tile_start.p, c.tile_beads.p,
-                                                       (float *)op.grid.p);
+    // offsets linear in x within a tile: no window may reach one from both ends
+    auto gather = n >= P + kTS ? k_spread_gather<true> : k_spread_gather<false>;
+    gather<<<nt * nt * nt, 64, 0, c.stream>>>(n, nt, P, (float)h, (float)alpha, (float)cn, tau_arg(c),
+                                              (const float4 *)c.wpos32.p, x, c.tile_start.p, c.tile_beads.p,
+                                              (float *)op.grid.p);
   } else {
   FSD_CUDA(cudaMemsetAsync(op.grid.p, 0, gbytes, c.stream));
   if (sizeof(T) == 4 && n % 4 == 0)
