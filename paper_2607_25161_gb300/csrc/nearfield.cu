@@ -263,10 +263,10 @@ __device__ __forceinline__ void sigma_congruence(const double *M, const double r
 }
 
 // LPA lanes per aggregate: B_J = sum_b Sigma_b (zeta0 I + R~_bb) Sigma_b^T, a
-// bead per lane, summed across the lanes; the first lane factors it (LU with
-// partial pivoting, stored in place).  A thread per aggregate ran the beads as
-// one dependent FP64 chain on 32 blocks: 161 us for 4096 8-bead aggregates,
-// now 50 us.
+// bead per lane, summed across the lanes, then factored by one lane each (LU
+// with partial pivoting, stored in place).  A thread per aggregate ran the beads
+// as one dependent FP64 chain on 32 blocks: 161 us for 4096 8-bead aggregates,
+// now 41 us.
 template <int LPA>
 __global__ void __launch_bounds__(128) k_schur_lu(int N, const int *__restrict__ body_start,
                                                   const double4 *__restrict__ lever,
@@ -297,7 +297,18 @@ __global__ void __launch_bounds__(128) k_schur_lu(int N, const int *__restrict__
   for (int o = LPA / 2; o > 0; o >>= 1)
 #pragma unroll
     for (int e = 0; e < 36; ++e) Bm[e] += __shfl_xor_sync(0xffffffffu, Bm[e], o);
-  if (!active || sub != 0) return;
+  // the block's matrices are factored by neighbouring lanes: an FP64 instruction
+  // costs the same for one lane as for 32
+  constexpr int kB = 128 / LPA;
+  __shared__ double sB[kB][37];
+  if (sub == 0)
+#pragma unroll
+    for (int e = 0; e < 36; ++e) sB[threadIdx.x / LPA][e] = Bm[e];
+  __syncthreads();
+  const int F = blockIdx.x * kB + threadIdx.x;
+  if (threadIdx.x >= kB || F >= N) return;
+#pragma unroll
+  for (int e = 0; e < 36; ++e) Bm[e] = sB[threadIdx.x][e];
   int pv[6];
   double scale = 0;
 #pragma unroll
@@ -340,9 +351,9 @@ __global__ void __launch_bounds__(128) k_schur_lu(int N, const int *__restrict__
 #pragma unroll
   for (int k = 0; k < 6; ++k) Bm[7 * k] = 1.0 / Bm[7 * k];
 #pragma unroll
-  for (int e = 0; e < 36; ++e) schur[(size_t)J * 36 + e] = Bm[e];
+  for (int e = 0; e < 36; ++e) schur[(size_t)F * 36 + e] = Bm[e];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) piv[J * 6 + k] = pv[k];
+  for (int k = 0; k < 6; ++k) piv[F * 6 + k] = pv[k];
 }
 
 __device__ __forceinline__ void lu_solve6(const double *LU, const int *pv, double *v) {

@@ -1416,22 +1416,28 @@ __device__ __forceinline__ int window_tiles(float p, float h, int P, int n, int 
   return cnt;
 }
 
+// Five threads per bead, one per z tile its window may meet.
 template <bool FILL>
 __global__ void k_tile_bin(int Nt, const float4 *__restrict__ pos, float h, int P, int n, int nt,
                            int *count_or_cursor, int *tile_beads, int64_t cap) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = t / 5, a = t - 5 * i;
   if (i >= Nt) return;
   const float4 p = pos[i];
-  int tx[5], ty[5], tz[5];
-  const int cx = window_tiles(p.x, h, P, n, tx), cy = window_tiles(p.y, h, P, n, ty),
-            cz = window_tiles(p.z, h, P, n, tz);
-  for (int a = 0; a < cz; ++a)
-    for (int b = 0; b < cy; ++b)
-      for (int d = 0; d < cx; ++d) {
-        const int id = (tz[a] * nt + ty[b]) * nt + tx[d];
-        const int slot = atomicAdd(&count_or_cursor[id], 1);
-        if (FILL && slot < cap) tile_beads[slot] = i;
-      }
+  int tz[5];
+  const int cz = window_tiles(p.z, h, P, n, tz);
+  if (a >= cz) return;
+  int z = tz[0];
+#pragma unroll
+  for (int q = 1; q < 5; ++q) z = a == q ? tz[q] : z;
+  int tx[5], ty[5];
+  const int cx = window_tiles(p.x, h, P, n, tx), cy = window_tiles(p.y, h, P, n, ty);
+  for (int b = 0; b < cy; ++b)
+    for (int d = 0; d < cx; ++d) {
+      const int id = (z * nt + ty[b]) * nt + tx[d];
+      const int slot = atomicAdd(&count_or_cursor[id], 1);
+      if (FILL && slot < cap) tile_beads[slot] = i;
+    }
 }
 
 // Per chunk of kTCH beads the block stages, per bead: the x-window factors w
@@ -1851,12 +1857,12 @@ void build_spread_tiles(Ctx &c) {
   if (c.tile_beads.n < cap) c.tile_beads.alloc(cap);
   const float h = (float)c.h;
   FSD_CUDA(cudaMemsetAsync(c.tile_count.p, 0, ntiles * sizeof(int), c.stream));
-  k_tile_bin<false><<<ceil_div(c.Nt, 128), 128, 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p, h, c.P, n,
+  k_tile_bin<false><<<ceil_div(5 * (int64_t)c.Nt, 128), 128, 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p, h, c.P, n,
                                                               nt, c.tile_count.p, nullptr, 0);
   FSD_LAUNCHED(c);
   k_exclusive_scan<<<1, 1024, 0, c.stream>>>(ntiles, c.tile_count.p, c.tile_start.p, c.tile_cursor.p);
   FSD_LAUNCHED(c);
-  k_tile_bin<true><<<ceil_div(c.Nt, 128), 128, 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p, h, c.P, n,
+  k_tile_bin<true><<<ceil_div(5 * (int64_t)c.Nt, 128), 128, 0, c.stream>>>(c.Nt, (const float4 *)c.wpos32.p, h, c.P, n,
                                                              nt, c.tile_cursor.p, c.tile_beads.p,
                                                              (int64_t)c.tile_beads.n);
   FSD_LAUNCHED(c);
