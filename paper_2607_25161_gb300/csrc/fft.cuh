@@ -31,8 +31,9 @@ struct alignas(2 * sizeof(T)) Cplx {
 };
 
 // Green's function operands of the z pass: the halved factors and 1/k^2 (in
-// (2 pi / L)^2).  Cubic box: green[4 m] by m = kx^2 + ky^2 + kz^2.  Lees-Edwards
-// box: gle[kx <= n/2][kz][ky][4] for the current offset, the physical wave vector
+// (2 pi / L)^2).  Cubic box: by m = kx^2 + ky^2 + kz^2, green[4 m] in FP64,
+// green[3 m] in FP32, where the division is cheap.  Lees-Edwards box:
+// gle[kx <= n/2][kz][ky][4] for the current offset, the physical wave vector
 // (kx, ky - tau kx, kz).
 template <typename T>
 struct ZGreen {
@@ -474,12 +475,18 @@ __device__ __forceinline__ int signed_k(int i, int n) { return i <= n / 2 ? i : 
 template <typename T, int n>
 __device__ __forceinline__ void green_at(const ZGreen<T> &g, int kx, int y, int z, T t[4]) {
   const int ky = signed_k(y, n), kz = signed_k(z, n);
-  const T *q = g.gle ? g.gle + 4 * (((int64_t)kx * n + z) * n + y) : g.green + 4 * (kx * kx + ky * ky + kz * kz);
+  const int m = kx * kx + ky * ky + kz * kz;
   if constexpr (sizeof(T) == 4) {
-    const float4 v = __ldg((const float4 *)q);
-    t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
+    if (g.gle) {
+      const float4 v = __ldg((const float4 *)g.gle + (((int64_t)kx * n + z) * n + y));
+      t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
+    } else {
+      const float *q = g.green + 3 * m;
+      t[0] = __ldg(q); t[1] = __ldg(q + 1); t[2] = __ldg(q + 2); t[3] = 1.f / (float)m;
+    }
   } else {
-    const double2 u = __ldg((const double2 *)q), v = __ldg((const double2 *)q + 1);
+    const double2 *q = (const double2 *)(g.gle ? g.gle + 4 * (((int64_t)kx * n + z) * n + y) : g.green + 4 * m);
+    const double2 u = __ldg(q), v = __ldg(q + 1);
     t[0] = u.x; t[1] = u.y; t[2] = v.x; t[3] = v.y;
   }
 }
@@ -615,7 +622,9 @@ __global__ void __launch_bounds__(Tile<T, R1, R2>::ZT)
     kk[1] = (T)((double)signed_k(ky, n) - tau * (double)kx);
     kyb = (T)((double)signed_k(my, n) - tau * (double)kx);
   }
-  for (int q = threadIdx.x / TP; q < n && ky < kend; q += NT / TP) {
+  for (int e = threadIdx.x; e < TP * n; e += NT) {
+    const int q = e / TP;
+    if (ky >= kend) continue;
     const int k1 = q % R1, k2 = q / R1, kz = k1 + R1 * k2;
     const int mz = kz == 0 ? 0 : n - kz;
     Cplx<T> *A = sm + t * L::LT + k1 * L::CS + k2;

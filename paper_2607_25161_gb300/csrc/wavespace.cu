@@ -1103,64 +1103,48 @@ __device__ __forceinline__ void read_out(const T *acc, int lane, int i, double *
 }
 
 // One warp per bead: u = h^3 sum W u_M, G_ab = h^3 sum 2 alpha W y_b u_D,a;
-// omega = (1/2) curl, e = sym G projected; added to the bead row of y.
-// PL: the six fields are planar [6][n^3] (from the fused FFT) instead of
-// interleaved [n^3][8].
-template <typename T, bool PL>
-__global__ void __launch_bounds__(256) k_interp(int Nt, const typename V4Of<T>::type *__restrict__ pos,
-                                                const T *__restrict__ grid, double *y, int n, int P,
-                                                T h, T alpha, T cnorm_h3, TauArg ta_, bool set) {
+// omega = (1/2) curl, e = sym G projected; to the bead row of y.  Planar FP32
+// fields [6][n^3] (grids whose side is no multiple of 4).
+__global__ void __launch_bounds__(256) k_interp(int Nt, const float4 *__restrict__ pos,
+                                                const float *__restrict__ grid, double *y, int n, int P,
+                                                float h, float alpha, float cnorm_h3, TauArg ta_, bool set) {
   const double tau = tau_of(ta_);
-  __shared__ T sw[8][3][kMaxP], sy[8][3][kMaxP];
+  __shared__ float sw[8][3][kMaxP], sy[8][3][kMaxP];
   __shared__ int si[8][3][kMaxP];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * (blockDim.x >> 5) + warp;
   if (i >= Nt) return;
-  const auto p = pos[i];
-  const T pc[3] = {p.x, p.y, p.z};
+  const float4 p = pos[i];
+  const float pc[3] = {p.x, p.y, p.z};
   for (int e = lane; e < 3 * P; e += 32) {
     int d = e / P, k = e - d * P;
-    int g0 = (int)floor_t<T>(pc[d] / h) - P / 2 + 1;
+    int g0 = (int)floorf(pc[d] / h) - P / 2 + 1;
     int g = g0 + k;
-    T yv = T(g) * h - pc[d];
-    sw[warp][d][k] = exp_t<T>(-alpha * yv * yv);
+    float yv = float(g) * h - pc[d];
+    sw[warp][d][k] = expf(-alpha * yv * yv);
     sy[warp][d][k] = yv;
     si[warp][d][k] = ((g % n) + n) % n;
   }
   __syncwarp();
   const int P3 = P * P * P;
-  const T ta = T(2) * alpha;
-  T acc[12];
+  const int64_t n3 = (int64_t)n * n * n;
+  const float ta = 2.f * alpha;
+  float acc[12];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = T(0);
+  for (int k = 0; k < 12; ++k) acc[k] = 0.f;
   for (int t = lane; t < P3; t += 32) {
     const int ix = t % P, iy = (t / P) % P, iz = t / (P * P);
-    const T W = sw[warp][0][ix] * sw[warp][1][iy] * sw[warp][2][iz];
-    const T y0 = sy[warp][0][ix], y1 = sy[warp][1][iy], y2 = sy[warp][2][iz];
-    T g6[6];
-    const int64_t gi = ((int64_t)si[warp][2][iz] * n + si[warp][1][iy]) * n + si[warp][0][ix];
-    if (PL) {
-      const int64_t n3 = (int64_t)n * n * n;
+    const float W = sw[warp][0][ix] * sw[warp][1][iy] * sw[warp][2][iz];
+    const float v[3] = {sy[warp][0][ix], sy[warp][1][iy], sy[warp][2][iz]};
+    const float *g = grid + ((int64_t)si[warp][2][iz] * n + si[warp][1][iy]) * n + si[warp][0][ix];
+    const float Wd = ta * W;
 #pragma unroll
-      for (int c = 0; c < 6; ++c) g6[c] = grid[c * n3 + gi];
-    } else {
-      load6<T>(grid + (gi << 3), g6);
+    for (int c = 0; c < 3; ++c) {
+      acc[c] += W * g[c * n3];
+      const float d = g[(3 + c) * n3];
+#pragma unroll
+      for (int e = 0; e < 3; ++e) acc[3 + 3 * c + e] += d * (Wd * v[e]);  // G_ce
     }
-    const T u0 = g6[0], u1 = g6[1], u2 = g6[2], d0 = g6[3], d1 = g6[4], d2 = g6[5];
-    acc[0] += W * u0;
-    acc[1] += W * u1;
-    acc[2] += W * u2;
-    T Wd = ta * W;
-    T w0 = Wd * y0, w1 = Wd * y1, w2 = Wd * y2;
-    acc[3] += d0 * w0;  // G_00
-    acc[4] += d0 * w1;  // G_01
-    acc[5] += d0 * w2;  // G_02
-    acc[6] += d1 * w0;  // G_10
-    acc[7] += d1 * w1;  // G_11
-    acc[8] += d1 * w2;  // G_12
-    acc[9] += d2 * w0;  // G_20
-    acc[10] += d2 * w1; // G_21
-    acc[11] += d2 * w2; // G_22
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1)
@@ -1677,25 +1661,28 @@ void build_wave(Ctx &c) {
   // Green table by m = kx^2 + ky^2 + kz^2
   const int hm = n / 2;
   const int mmax = 3 * hm * hm;
-  // two-factor passes: halved factors and 1/m
+  // two-factor passes: halved factors, in FP64 with 1/m
   const bool two = fft_ops<double>(n) != nullptr;
-  const int gw = two ? 4 : 3;
-  std::vector<double> gr((size_t)gw * (mmax + 1), 0.0);
-  const double n3 = (double)n * n * n;
-  for (int m = 1; m <= mmax; ++m) {
-    double k = 2.0 * kPi * std::sqrt((double)m) / c.L;
-    double k2 = k * k;
-    double e = -k2 / (4.0 * c.xi * c.xi) + k2 / (2.0 * c.alpha);
-    double A = (1.0 + k2 / (4.0 * c.xi * c.xi)) * std::exp(e) / (c.eta * k2) / n3;
-    double fm = j0h(k * c.a), fd = fDh(k * c.a);
-    const double sc = two ? 0.5 * A : A;
-    gr[(size_t)gw * m] = sc * fm * fm;
-    gr[(size_t)gw * m + 1] = sc * fm * fd;
-    gr[(size_t)gw * m + 2] = sc * fd * fd;
-    if (two) gr[(size_t)gw * m + 3] = 1.0 / m;
+  for (int gw : {3, 4}) {
+    if (gw == 4 && !two) break;
+    std::vector<double> gr((size_t)gw * (mmax + 1), 0.0);
+    const double n3 = (double)n * n * n;
+    for (int m = 1; m <= mmax; ++m) {
+      double k = 2.0 * kPi * std::sqrt((double)m) / c.L;
+      double k2 = k * k;
+      double e = -k2 / (4.0 * c.xi * c.xi) + k2 / (2.0 * c.alpha);
+      double A = (1.0 + k2 / (4.0 * c.xi * c.xi)) * std::exp(e) / (c.eta * k2) / n3;
+      double fm = j0h(k * c.a), fd = fDh(k * c.a);
+      const double sc = two ? 0.5 * A : A;
+      double *g = gr.data() + (size_t)gw * m;
+      g[0] = sc * fm * fm;
+      g[1] = sc * fm * fd;
+      g[2] = sc * fd * fd;
+      if (gw == 4) g[3] = 1.0 / m;
+    }
+    if (gw == 4 || !two) upload(c.op64.green, gr);
+    if (gw == 3) upload(c.op32.green, gr);
   }
-  upload(c.op64.green, gr);
-  upload(c.op32.green, gr);
   // Brownian wave-field scales (Sec. 2.2, Eq. UBff): the random field xi(k)
   // becomes f(k) sqrt(H(k)/(eta k^2)) / (sqrt(V) W^(k)) (I - k k) xi(k), the
   // analytic square root of the wave part once the interpolation's Gaussian
@@ -1828,8 +1815,9 @@ static void wave_tail(Ctx &c, OpData<T> &op, Cx<T> *spec, double *y, bool set) {
                                                             (const float *)op.gout.p, y, n, P, (float)h,
                                                             (float)alpha, (float)(cn * h3), tau_arg(c), set);
   else if (planar)
-    k_interp<T, true><<<ceil_div(c.Nt, bead_warps(c)), 32 * bead_warps(c), 0, c.stream>>>(c.Nt, posp<T>(c), op.gout.p, y, n, P,
-                                                              h, alpha, (T)(cn * h3), tau_arg(c), set);
+    k_interp<<<ceil_div(c.Nt, bead_warps(c)), 32 * bead_warps(c), 0, c.stream>>>(
+        c.Nt, (const float4 *)c.wpos32.p, (const float *)op.gout.p, y, n, P, (float)h, (float)alpha,
+        (float)(cn * h3), tau_arg(c), set);
   else
     k_interp_rows<T><<<ceil_div(c.Nt, bead_warps(c)), 32 * bead_warps(c), 0, c.stream>>>(c.Nt, posp<T>(c), op.gout.p, y, n,
                                                               P, h, alpha, (T)(cn * h3),
@@ -2121,7 +2109,7 @@ NaLayout na_layout(int n, int nb) {
   l.gout = o;
   o += na_round((size_t)8 * n * n * n * sizeof(float));
   l.green = o;
-  o += na_round((size_t)4 * (3 * (n / 2) * (n / 2) + 1) * sizeof(float));
+  o += na_round((size_t)3 * (3 * (n / 2) * (n / 2) + 1) * sizeof(float));
   l.tw = o;
   o += na_round((size_t)2 * n * sizeof(float));
   l.pos = o;
@@ -2147,7 +2135,7 @@ __global__ void k_na_tables(int n, int R2, float *tw, float *green, int mmax, do
   const double n3 = (double)n * n * n;
   for (int m = t0; m <= mmax; m += stride) {
     if (m == 0) {
-      green[0] = green[1] = green[2] = green[3] = 0.f;
+      green[0] = green[1] = green[2] = 0.f;
       continue;
     }
     const double k = 2.0 * kPi * sqrt((double)m) / L, k2 = k * k;
@@ -2157,10 +2145,9 @@ __global__ void k_na_tables(int n, int R2, float *tw, float *green, int mmax, do
     const double fm = z < 1e-3 ? 1.0 - z * z / 6.0 + z * z * z * z / 120.0 : sin(z) / z;
     const double fd = z < 1e-2 ? 1.0 - z * z / 10.0 + z * z * z * z / 280.0
                                : 3.0 * (sin(z) - z * cos(z)) / (z * z * z);
-    green[4 * m] = (float)(0.5 * A * fm * fm);
-    green[4 * m + 1] = (float)(0.5 * A * fm * fd);
-    green[4 * m + 2] = (float)(0.5 * A * fd * fd);
-    green[4 * m + 3] = (float)(1.0 / m);
+    green[3 * m] = (float)(0.5 * A * fm * fm);
+    green[3 * m + 1] = (float)(0.5 * A * fm * fd);
+    green[3 * m + 2] = (float)(0.5 * A * fd * fd);
   }
 }
 
@@ -2278,7 +2265,7 @@ extern "C" fsd_status fsd_apply_wave_noalloc(int64_t n_beads, const double *bead
     k_interp_brick<<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3, TauArg(),
                                               true);
   else
-    k_interp<float, true><<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3,
+    k_interp<<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, gout, y, n, P, (float)h, (float)alpha, cnh3,
                                                        TauArg(), true);
   k_na_stage_out<<<(nb + 127) / 128, 128, 0, st>>>(nb, y, out);
   if (cudaGetLastError() != cudaSuccess) return FSD_ECUDA;
