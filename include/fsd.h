@@ -112,7 +112,7 @@ enum {
                               On this part FP64 runs at 1/74 of the FP32 rate
                               and the FP64 Gram-Schmidt passes are ALU-bound;
                               the FP32 basis takes the 32768-bead step from
-                              ~66 to ~61 ms at the same iteration count and
+                              47.7 to 43.3 ms at the same iteration count and
                               accuracy */
 };
 

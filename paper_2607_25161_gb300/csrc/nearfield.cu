@@ -125,7 +125,7 @@ __device__ __forceinline__ void min_image(double &d0, double &d1, double &d2, do
 // Bound by FP64 arithmetic (a logarithm, a square root and the divisions).
 // A thread per bead walked its pairs one after the other, a dependent FP64
 // chain with a third of the lanes idle, and wrote 288-byte strides: with the
-// diagonal blocks 241 us for the 101 632 pairs of 32768 beads, now 73 + 42 us.
+// diagonal blocks 241 us for the 101 632 pairs of 32768 beads, now 57 + 40 us.
 constexpr int kLP = 64;  // pairs per block
 __global__ void __launch_bounds__(kLP) k_lub_pairs(
     int Nt, int nnz, const double4 *__restrict__ pos, const int *__restrict__ lnbr, int lcap,

@@ -1,7 +1,7 @@
 // Wave-space part of the PSE mobility (Sec. 2.2, Eq. UBff split; Sec. 3.2
 // grid rule): Gaussian spreading of the force and force-dipole densities, a
-// hand-written shared-memory mixed-radix 3D FFT with the Green's function
-// scaling fused into the z pass, and interpolation of the velocity and
+// hand-written 3D FFT with the Green's function scaling between the z pass's
+// two transforms, and interpolation of the velocity and
 // velocity gradient.
 //
 // Spreading.  FP32 (the Krylov operator): grid-centric, k_spread_gather.
@@ -18,7 +18,7 @@
 // three complex fields g_p + i g_(p+3), with the Green's function between the
 // forward and inverse z transforms; the inverse leaves bricked or planar velocity fields
 // (FP32) or interleaved ones [n^3][8] (FP64).  On the 32768-bead
-// benchmark (n = 144, FP32) the five passes take 0.165 ms against 0.243 for
+// benchmark (n = 144, FP32) the five passes take 0.151 ms against 0.243 for
 // the fused plane kernels and staged z pass they replaced, 0.62 against 1.31
 // ms at n = 216 and, in FP64, 0.71 against 1.08 ms at n = 96.  Other sizes
 // take the staged plan: half spectra [6][n][n][n/2 + 1] and interleaved
@@ -1425,16 +1425,18 @@ __global__ void k_tile_bin(int Nt, const float4 *__restrict__ pos, float h, int 
 }
 
 // Per chunk of kTCH beads the block stages, per bead: the x-window factors w
-// and their products with the offset, w (g h - p), for the tile's 8 x
-// points (the dipole term's x factor); (w, offset) pairs for its 8 y and 8 z
+// for the tile's 8 x points, with their products with the offset, w (g h - p)
+// (the dipole term's x factor), or with LIN the first point's offset, from
+// which a row forms them; (w, offset) pairs for its 8 y and 8 z
 // points; the twelve scaled moments; and 8-bit masks of the tile's y and z
 // rows its window reaches.  Each thread then iterates over exactly the
 // beads whose window covers its (y, z) row (a bit mask over the chunk, from
 // sixteen warp ballots), so a warp runs the largest count among its rows
 // instead of every bead listed for the tile.  Bound by instruction issue: the
 // 72 multiply-adds of a (bead, row) are taken two x points at a time in one
-// instruction (same rounding), 0.152 -> 0.130 ms per application on 32768
-// beads at n = 144, with 10 blocks per SM (12 spill, 0.152; 8: 0.140).
+// instruction (same rounding): 0.152 -> 0.127 ms per application on 32768
+// beads at n = 144, with 10 blocks per SM (12 spill, 0.152; 8: 0.140); 0.123
+// with LIN below.
 template <bool LIN>
 __global__ void __launch_bounds__(64, 10) k_spread_gather(int n, int nt, int P, float h, float alpha,
                                                       float cnorm, TauArg ta_,
