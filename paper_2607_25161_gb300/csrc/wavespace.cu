@@ -1230,8 +1230,10 @@ __global__ void __launch_bounds__(256) k_interp_rows(int Nt, const typename V4Of
 // four x points of one of four neighbouring bricks along x: its x and y weights
 // stay in registers, it steps through the window's bricks along z with six
 // 16-byte loads each, and a quarter of a warp request is one 128-byte line.
-// Bound by the L1 pipe and the lines it misses (about half: each point is in
-// 19 windows on average, but few of them at once): with rows of the plain [z][y][x] layout a request
+// Bound by the latency of the lines its L1 misses (about half: each point is
+// in 19 windows on average, but few of them at once; L1 pipe 48 %, issue 51 %
+// busy, and more warps with fewer registers were slower).  With rows of the
+// plain [z][y][x] layout a request
 // touched eight rows of one or two lines each, twice the lines, and spent as
 // many instructions again on splitting an item index and reading weights
 // (0.170 ms per application on 32768 beads, n = 144, P = 12; 0.157 with
@@ -2081,8 +2083,8 @@ template void launch_brownian_wave<double>(Ctx &, const double *, uint64_t, uint
 // that loads this library and stays there until the process exits.  All
 // calls share it: two calls whose GPU work overlaps race on it, so a caller
 // must order them (one stream, or events).  Each call rewrites the parts it
-// reads before reading them and zeroes the density grids and the staged
-// output before accumulating into them.  Host code cannot use the array's
+// reads before reading them and zeroes the density grids before
+// accumulating into them.  Host code cannot use the array's
 // name as a device address: each call looks the address up in the current
 // device context (cudaGetSymbolAddress), so a device reset or another
 // context on the same device never leaves a stale address behind.
@@ -2124,22 +2126,43 @@ NaLayout na_layout(int n, int nb) {
   return l;
 }
 
-// Twiddles of the transform and the Green's table (same formulas as build_wave).
-__global__ void k_na_tables(int n, int R2, float *tw, float *green, int mmax, double L, double xi,
-                            double alpha, double a, double eta) {
-  const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
-  const int stride = gridDim.x * blockDim.x;
-  for (int t = t0; t < n; t += stride) {
+// Everything the spreading and the transforms read, in one launch of three
+// kinds of blocks: the twiddles and the Green's table (same formulas as
+// build_wave), 32 entries per block; the beads' wrapped positions and moments
+// in the staged layout, 32 beads per block; and the zeroing of the density
+// grids.  The tables' FP64 functions bound it, and an SM's FP64 pipe takes one
+// warp of them at a time, so each block has one such warp and the blocks spread
+// over the SMs: as two kernels of 8 and nb / 128 blocks and a memset, a call of
+// 700 beads on 40^3 took 82 us, now 66.
+constexpr int kNaT = 128;
+struct NaBlocks {
+  int tw, green, beads, zero;  // blocks of each kind
+};
+
+__global__ void __launch_bounds__(kNaT) k_na_prepare(NaBlocks nblk, int n, int R2, float *tw, float *green,
+                                                     int mmax, double L, double xi, double alpha, double a,
+                                                     double eta, int nb, const double *__restrict__ pos,
+                                                     const double *__restrict__ in, float4 *pos4, double *x,
+                                                     float4 *grid, int64_t nquads) {
+  const int lane = threadIdx.x;
+  int b = blockIdx.x;
+  if (b < nblk.tw) {
+    const int t = 32 * b + lane;
+    if (lane >= 32 || t >= n) return;
     const double ang = -2.0 * kPi * (t / R2) * (t % R2) / (double)n;
     tw[2 * t] = (float)cos(ang);
     tw[2 * t + 1] = (float)sin(ang);
+    return;
   }
-  const double n3 = (double)n * n * n;
-  for (int m = t0; m <= mmax; m += stride) {
+  b -= nblk.tw;
+  if (b < nblk.green) {
+    const int m = 32 * b + lane;
+    if (lane >= 32 || m > mmax) return;
     if (m == 0) {
       green[0] = green[1] = green[2] = 0.f;
-      continue;
+      return;
     }
+    const double n3 = (double)n * n * n;
     const double k = 2.0 * kPi * sqrt((double)m) / L, k2 = k * k;
     const double e = -k2 / (4.0 * xi * xi) + k2 / (2.0 * alpha);
     const double A = (1.0 + k2 / (4.0 * xi * xi)) * exp(e) / (eta * k2) / n3;
@@ -2150,27 +2173,31 @@ __global__ void k_na_tables(int n, int R2, float *tw, float *green, int mmax, do
     green[3 * m] = (float)(0.5 * A * fm * fm);
     green[3 * m + 1] = (float)(0.5 * A * fm * fd);
     green[3 * m + 2] = (float)(0.5 * A * fd * fd);
+    return;
   }
-}
-
-// Bead positions (wrapped into [0, L)) and moments into the staged layout;
-// the staged output rows are zeroed (interpolation accumulates into them).
-__global__ void k_na_stage_in(int nb, const double *__restrict__ pos, const double *__restrict__ in,
-                              double L, float4 *pos4, double *x, double *y) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nb) return;
-  float p[3];
-  for (int d = 0; d < 3; ++d) {
-    double v = pos[3 * (size_t)i + d];
-    v -= L * floor(v / L);
-    if (v >= L) v -= L;
-    if (v < 0) v = 0;
-    p[d] = (float)v;
+  b -= nblk.green;
+  if (b < nblk.beads) {
+    const int i0 = 32 * b, nc = min(32, nb - i0);
+    for (int k = lane; k < LDB * nc; k += kNaT) {
+      const int i = i0 + k / LDB, c = k % LDB;
+      x[(size_t)i * LDB + c] = c < 11 ? in[(size_t)i * 11 + c] : 0.0;
+    }
+    if (lane >= nc) return;
+    const int i = i0 + lane;
+    float p[3];
+    for (int d = 0; d < 3; ++d) {  // wrapped into [0, L)
+      double v = pos[3 * (size_t)i + d];
+      v -= L * floor(v / L);
+      if (v >= L) v -= L;
+      if (v < 0) v = 0;
+      p[d] = (float)v;
+    }
+    pos4[i] = make_float4(p[0], p[1], p[2], 0.f);
+    return;
   }
-  pos4[i] = make_float4(p[0], p[1], p[2], 0.f);
-  for (int k = 0; k < 11; ++k) x[(size_t)i * LDB + k] = in[(size_t)i * 11 + k];
-  x[(size_t)i * LDB + 11] = 0.0;
-  for (int k = 0; k < LDB; ++k) y[(size_t)i * LDB + k] = 0.0;
+  b -= nblk.beads;
+  for (int64_t q = (int64_t)b * kNaT + lane; q < nquads; q += (int64_t)nblk.zero * kNaT)
+    grid[q] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 __global__ void k_na_stage_out(int nb, const double *__restrict__ y, double *out) {
@@ -2242,10 +2269,14 @@ extern "C" fsd_status fsd_apply_wave_noalloc(int64_t n_beads, const double *bead
   const FftOps<float> *f = fft_ops<float>(n);  // built for every accepted grid
   if (!f) return FSD_EINVAL;
   const int hm = n / 2, mmax = 3 * hm * hm;
-  k_na_tables<<<8, 256, 0, st>>>(n, f->R2, tw, green, mmax, L, xi, alpha, a, eta);
-  k_na_stage_in<<<(nb + 127) / 128, 128, 0, st>>>(nb, bead_pos, in, L, pos4, x, y);
-  if (cudaMemsetAsync(gridp, 0, (size_t)6 * n * n * n * sizeof(float), st) != cudaSuccess)
-    return FSD_ECUDA;
+  const int64_t nquads = (int64_t)6 * n * n * n / 4;  // n is even
+  NaBlocks nblk;
+  nblk.tw = (n + 31) / 32;
+  nblk.green = (mmax + 32) / 32;
+  nblk.beads = (nb + 31) / 32;
+  nblk.zero = (int)std::min<int64_t>((nquads + 4 * kNaT - 1) / (4 * kNaT), 304);
+  k_na_prepare<<<nblk.tw + nblk.green + nblk.beads + nblk.zero, kNaT, 0, st>>>(
+      nblk, n, f->R2, tw, green, mmax, L, xi, alpha, a, eta, nb, bead_pos, in, pos4, x, (float4 *)gridp, nquads);
   const double cn = std::pow(alpha / kPi, 1.5);
   if (n % 4 == 0)
     k_spread_v4<<<(nb + 7) / 8, 256, 0, st>>>(nb, pos4, x, gridp, n, P, (float)h, (float)alpha, (float)cn,
