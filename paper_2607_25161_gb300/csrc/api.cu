@@ -590,7 +590,7 @@ static void setup_impl(Ctx &c, int64_t n_beads, const double *bead_pos, const in
   c.wpos64.alloc(4 * (size_t)Nt);
   c.wpos32.alloc(4 * (size_t)Nt);
   if (c.overlap) c.yw.alloc((size_t)LDB * Nt);
-  FSD_CUDA(cudaMemcpy(c.body_start.p, c.h_body_start.data(), (N + 1) * sizeof(int), cudaMemcpyHostToDevice));
+  upload(c, c.body_start.p, c.h_body_start.data(), N + 1);
   {
     // lanes per aggregate of the aggregate-row kernels: the power of two
     // (4..32) that covers the largest aggregate
@@ -599,12 +599,12 @@ static void setup_impl(Ctx &c, int64_t n_beads, const double *bead_pos, const in
     c.body_lanes = 4;
     while (c.body_lanes < 32 && c.body_lanes < mb) c.body_lanes *= 2;
   }
-  FSD_CUDA(cudaMemcpy(c.bead_body.p, bead_body.data(), Nt * sizeof(int), cudaMemcpyHostToDevice));
-  FSD_CUDA(cudaMemcpy(c.perm_bead.p, c.h_perm_bead.data(), Nt * sizeof(int), cudaMemcpyHostToDevice));
-  FSD_CUDA(cudaMemcpy(c.perm_body.p, c.h_perm_body.data(), N * sizeof(int), cudaMemcpyHostToDevice));
-  FSD_CUDA(cudaMemcpy(c.X.p, Xi.data(), Xi.size() * sizeof(double), cudaMemcpyHostToDevice));
-  FSD_CUDA(cudaMemcpy(c.q.p, qi.data(), qi.size() * sizeof(double), cudaMemcpyHostToDevice));
-  FSD_CUDA(cudaMemcpy(c.rbody.p, rbi.data(), rbi.size() * sizeof(double), cudaMemcpyHostToDevice));
+  upload(c, c.bead_body.p, bead_body.data(), Nt);
+  upload(c, c.perm_bead.p, c.h_perm_bead.data(), Nt);
+  upload(c, c.perm_body.p, c.h_perm_body.data(), N);
+  upload(c, c.X.p, Xi.data(), Xi.size());
+  upload(c, c.q.p, qi.data(), qi.size());
+  upload(c, c.rbody.p, rbi.data(), rbi.size());
   // neighbour capacities from the mean density (grown on overflow)
   const double dens = Nt / (L * L * L);
   const double expect = dens * 4.0 / 3.0 * kPi * c.rc * c.rc * c.rc;
@@ -623,8 +623,8 @@ static void setup_impl(Ctx &c, int64_t n_beads, const double *bead_pos, const in
   c.piv.alloc((size_t)N * 6);
   c.fnf.alloc((size_t)Nt * 6);
   c.snf.alloc((size_t)Nt * 5);
-  FSD_CUDA(cudaMemset(c.fnf.p, 0, (size_t)Nt * 6 * sizeof(double)));
-  FSD_CUDA(cudaMemset(c.snf.p, 0, (size_t)Nt * 5 * sizeof(double)));
+  FSD_CUDA(cudaMemsetAsync(c.fnf.p, 0, (size_t)Nt * 6 * sizeof(double), c.stream));
+  FSD_CUDA(cudaMemsetAsync(c.snf.p, 0, (size_t)Nt * 5 * sizeof(double), c.stream));
   const int mm = std::max(c.m, c.m_in);
   // V: FP64 GMRES and the Lanczos square roots (at most mm + 1 vectors);
   // with FSD_FLAG_FP32_KRYLOV the mixed solve's inner GMRES keeps its bases
@@ -649,7 +649,7 @@ static void setup_impl(Ctx &c, int64_t n_beads, const double *bead_pos, const in
   c.partial.alloc(std::max<int64_t>((int64_t)64 * kDotPartials, cgs_partial_size(c.nunk, mm + 1, c.num_sms)));
   c.hcol.alloc(512);
   c.cgs_ticket.alloc(1);
-  FSD_CUDA(cudaMemset(c.cgs_ticket.p, 0, sizeof(unsigned)));
+  FSD_CUDA(cudaMemsetAsync(c.cgs_ticket.p, 0, sizeof(unsigned), c.stream));
   FSD_CUDA(cudaMallocHost(&c.h_pinned, 512 * sizeof(double)));
   build_real_table(c);
   build_wave(c);

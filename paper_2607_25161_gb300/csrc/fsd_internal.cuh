@@ -249,6 +249,13 @@ struct Ctx {
   double tuned_ms = 0.0;  // operator time measured by the autotuner (0: not tuned)
 };
 
+// Host array -> device on the context's stream; the source may go on return.
+template <typename T>
+void upload(Ctx &c, T *dst, const T *src, size_t count) {
+  FSD_CUDA(cudaMemcpyAsync(dst, src, count * sizeof(T), cudaMemcpyHostToDevice, c.stream));
+  FSD_CUDA(cudaStreamSynchronize(c.stream));
+}
+
 // ------------------------------------------------------ Lees-Edwards box
 // Nearest image of a displacement in the sheared periodic box (lattice
 // (L,0,0), (tilt,L,0), (0,0,L)): wrap y first, shifting x by the offset, then

@@ -608,7 +608,10 @@ static void ensure_cache(Ctx &c) {
   c.gcache = new GraphCache();
   GraphCache &gc = *c.gcache;
   gc.state.alloc(1);
-  FSD_CUDA(cudaMemset(gc.state.p, 0, sizeof(GState)));
+  // on the context's stream, as every clear and upload of a context: the legacy
+  // stream is not ordered with it, and a clear queued there behind another
+  // system's graph could run in the middle of this context's solve
+  FSD_CUDA(cudaMemsetAsync(gc.state.p, 0, sizeof(GState), c.stream));
   FSD_CUDA(cudaMallocHost(&gc.h_state, sizeof(GState)));
   gc.vin.alloc(c.nunk);
   gc.zf.alloc(c.nunk);

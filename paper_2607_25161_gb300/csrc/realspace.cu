@@ -171,12 +171,10 @@ void build_real_table(Ctx &c) {
   double w1 = wave_phi(q, 0, 0.0), w2 = wave_phi(q, 4, 0.0);
   double self[3] = {mt - 2.0 * w1, mr + 2.5 * w2, ms + 3.0 * w2};
   c.op64.table.alloc(tab.size());
-  FSD_CUDA(cudaMemcpy(c.op64.table.p, tab.data(), tab.size() * sizeof(double),
-                      cudaMemcpyHostToDevice));
+  upload(c, c.op64.table.p, tab.data(), tab.size());
   std::vector<float> tabf(tab32.begin(), tab32.end());
   c.op32.table.alloc(tabf.size());
-  FSD_CUDA(cudaMemcpy(c.op32.table.p, tabf.data(), tabf.size() * sizeof(float),
-                      cudaMemcpyHostToDevice));
+  upload(c, c.op32.table.p, tabf.data(), tabf.size());
   for (int i = 0; i < 3; ++i) {
     c.op64.self_real[i] = self[i];
     c.op32.self_real[i] = (float)self[i];

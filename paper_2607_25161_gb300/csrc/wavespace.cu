@@ -1630,10 +1630,10 @@ static double fDh(double z) {
 }
 
 template <typename T>
-static void upload(DBuf<T> &buf, const std::vector<double> &v) {
+static void upload_as(Ctx &c, DBuf<T> &buf, const std::vector<double> &v) {
   std::vector<T> tv(v.begin(), v.end());
   buf.alloc(tv.size());
-  FSD_CUDA(cudaMemcpy(buf.p, tv.data(), tv.size() * sizeof(T), cudaMemcpyHostToDevice));
+  upload(c, buf.p, tv.data(), tv.size());
 }
 
 void build_wave(Ctx &c) {
@@ -1660,8 +1660,8 @@ void build_wave(Ctx &c) {
   } else {
     make_plan(n, &tw, true);
   }
-  upload(c.op64.twiddle, tw);
-  upload(c.op32.twiddle, tw);
+  upload_as(c, c.op64.twiddle, tw);
+  upload_as(c, c.op32.twiddle, tw);
   // Green table by m = kx^2 + ky^2 + kz^2
   const int hm = n / 2;
   const int mmax = 3 * hm * hm;
@@ -1684,8 +1684,8 @@ void build_wave(Ctx &c) {
       g[2] = sc * fd * fd;
       if (gw == 4) g[3] = 1.0 / m;
     }
-    if (gw == 4 || !two) upload(c.op64.green, gr);
-    if (gw == 3) upload(c.op32.green, gr);
+    if (gw == 4 || !two) upload_as(c, c.op64.green, gr);
+    if (gw == 3) upload_as(c, c.op32.green, gr);
   }
   // Brownian wave-field scales (Sec. 2.2, Eq. UBff): the random field xi(k)
   // becomes f(k) sqrt(H(k)/(eta k^2)) / (sqrt(V) W^(k)) (I - k k) xi(k), the
@@ -1701,8 +1701,8 @@ void build_wave(Ctx &c) {
     bt[2 * m] = sc * j0h(k * c.a);
     bt[2 * m + 1] = sc * fDh(k * c.a);
   }
-  upload(c.op64.btab, bt);
-  upload(c.op32.btab, bt);
+  upload_as(c, c.op64.btab, bt);
+  upload_as(c, c.op32.btab, bt);
 }
 
 template <typename T>
