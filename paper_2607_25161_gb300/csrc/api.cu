@@ -804,6 +804,10 @@ static StepMark graph_step_begin(Ctx &c, const double *ft_user, double shear, bo
 static fsd_status graph_step_end(Ctx &c, const StepMark &mk, fsd_stats *stats) {
   KStats ks;
   const double rel = graph_finish(c, ks);
+  if (rel < 0.0) {
+    c.last_error = "the solver state was cleared during the solve";
+    return FSD_ENUMERIC;
+  }
   c.have_prev = true;
   const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - mk.t0).count();
   fill_stats(c, stats, ks, rel, ms);

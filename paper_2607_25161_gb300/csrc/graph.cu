@@ -30,6 +30,7 @@ struct GState {
   int m;          // restart length of the running GMRES
   int outer;      // refinement sweeps (mixed)
   int status;     // bit 0: NaN in the Krylov process
+  int begun;      // set by k_g_reset alone: the end state is this solve's
   int xnz;        // the iterate x is nonzero (its residual needs A x)
   int cont;       // the Arnoldi loop goes on
   int ky;         // length of the least-squares solution y
@@ -98,6 +99,7 @@ __global__ void k_g_reset(GState *s, int m, int cyc_max, int max_total, double t
   s->m = m;
   s->outer = 0;
   s->status = 0;
+  s->begun = 1;
   s->xnz = xnz;
   s->cont = 0;
   s->ky = 0;
@@ -716,13 +718,15 @@ void graph_launch(Ctx &c, const GraphRun &o) {
 }
 
 // Wait for the launched graph; fill the Krylov statistics; return the final
-// relative residual.
+// relative residual, negative when the solver state is not one that a solve left.
 double graph_finish(Ctx &c, KStats &st) {
   GraphCache &gc = *c.gcache;
   FSD_CUDA(cudaStreamSynchronize(c.stream));
   const GraphEntry &e = gc.entries[c.graph_pending];
   const GState &s = *gc.h_state;
   if (s.status & 1) throw Invalid{"NaN in the Krylov process"};
+  // a state cleared under way would read as b = 0, solved with no residual
+  if (s.begun != 1) return -1.0;
   st.iters = s.total;
   st.m64 = s.mv64;
   st.m32 = s.mv32;
