@@ -689,9 +689,9 @@ static void fill_stats(Ctx &c, fsd_stats *st, const KStats &k, double rel, doubl
 }
 
 static fsd_status check_flags(Ctx &c) {
-  FSD_CUDA(cudaMemcpyAsync(c.h_flags, c.flags.p, 8 * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+  FSD_CUDA(cudaMemcpyAsync(c.h_flags, c.flags.p, kFlags * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
   FSD_CUDA(cudaStreamSynchronize(c.stream));
-  if (c.h_flags[3]) {
+  if (c.h_flags[kSingular]) {
     c.last_error = "singular per-aggregate 6x6 preconditioner block";
     return FSD_ENUMERIC;
   }
@@ -729,7 +729,7 @@ static fsd_status solve_internal(Ctx &c, const double *ft_user, double shear, do
   FSD_CUDA(cudaMemsetAsync(c.flags.p + 6, 0, sizeof(int), c.stream));
   k_nan_check<<<c.num_sms, 256, 0, c.stream>>>(vel_int, 6 * (int64_t)c.N, c.flags.p + 6);
   FSD_LAUNCHED(c);
-  FSD_CUDA(cudaMemcpyAsync(c.h_flags, c.flags.p, 8 * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+  FSD_CUDA(cudaMemcpyAsync(c.h_flags, c.flags.p, kFlags * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
   FSD_CUDA(cudaStreamSynchronize(c.stream));
   double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count() + t0_ms;
   fill_stats(c, stats, ks, rel, ms);
@@ -816,7 +816,7 @@ static fsd_status graph_step_end(Ctx &c, const StepMark &mk, fsd_stats *stats) {
     c.last_error = "non-finite aggregate velocity";
     return FSD_ENUMERIC;
   }
-  if (c.h_flags[3]) {
+  if (c.h_flags[kSingular]) {
     c.last_error = "singular per-aggregate 6x6 preconditioner block";
     return FSD_ENUMERIC;
   }

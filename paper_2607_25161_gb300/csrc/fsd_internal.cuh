@@ -34,7 +34,9 @@ constexpr int tab_stride() {
   return tab_coef<T>() * 8 + 4;
 }
 constexpr int BLK = 36;     // 6x6 block
-constexpr int kFlags = 12;  // words of Ctx::flags
+constexpr int kFlags = 13;     // words of Ctx::flags
+constexpr int kSearchFlags = 12;  // the first of them, cleared by the pair search
+constexpr int kSingular = 12;     // singular LU: cleared and set by build_lubrication alone
 
 // ------------------------------------------------------------------ errors
 struct CudaError {
@@ -195,8 +197,9 @@ struct Ctx {
   int cap = 0, lcap = 0, ncell = 1;
   DBuf<int> nbr, ncnt, lnbr, lcnt;
   DBuf<int> cell_count, cell_start, cell_beads, cell_cursor, cell_id;
-  // [0] nbr overflow, [1] lub overflow, [2] overlap, [3] singular LU, [4] / [5] largest counts on
-  // overflow, [6] NaN, [8..11] total mobility and lubrication neighbours (two 64-bit sums)
+  // [0] nbr overflow, [1] lub overflow, [2] overlap, [4] / [5] largest counts on overflow,
+  // [6] NaN, [8..11] total mobility and lubrication neighbours (two 64-bit sums),
+  // [kSingular] singular LU
   DBuf<int> flags;
   int *h_flags = nullptr;  // pinned
   // ---- lubrication BSR (rows = beads; diagonal separate)

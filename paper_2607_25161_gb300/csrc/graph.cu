@@ -666,7 +666,7 @@ static GraphEntry &build_entry(Ctx &c, const GraphRun &o, const GraphKey &k) {
       launch_integrate(c, c.t1.p, o.dt, o.shear);
       launch_wrap_positions(c);
     }
-    FSD_CUDA(cudaMemcpyAsync(c.h_flags, c.flags.p, 8 * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+    FSD_CUDA(cudaMemcpyAsync(c.h_flags, c.flags.p, kFlags * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
     FSD_CUDA(cudaMemcpyAsync(gc.h_state, gc.state.p, sizeof(GState), cudaMemcpyDeviceToHost, c.stream));
     e.l_top += c.launches - l1;
     cap_end(c);

@@ -177,7 +177,8 @@ __global__ void __launch_bounds__(kLP) k_lub_pairs(
 // and the preconditioner's (pairs closer than r_p only) from the pair records; R_ii has 15 distinct entries.
 __global__ void __launch_bounds__(kLP) k_lub_diag(int Nt, const int *__restrict__ brow,
                                                   const PairRec *__restrict__ rec, double *bdiag64,
-                                                  double *pdiag) {
+                                                  double *pdiag, int *flags) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) flags[kSingular] = 0;  // the LUs of this geometry follow
   __shared__ double sb[kLP][37];
   const int i0 = blockIdx.x * kLP, i = i0 + threadIdx.x;
   double acc[2][15];
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(128) k_schur_lu(int N, const int *__restrict__
         p = rr;
       }
     if (best <= 1e-14 * scale || !(best == best)) {
-      atomicOr(&flags[3], 1);
+      atomicOr(&flags[kSingular], 1);
       Bm[6 * k + k] = (best == best && scale > 0) ? 1e-14 * scale : 1.0;
       p = k;
     }
@@ -1038,7 +1039,7 @@ void build_lubrication(Ctx &c) {
     FSD_LAUNCHED(c);
   }
   k_lub_diag<<<ceil_div(Nt, kLP), kLP, 0, c.stream>>>(Nt, c.brow.p, rec, lanczos ? c.bdiag.p : nullptr,
-                                                     c.pdiag.p);
+                                                     c.pdiag.p, c.flags.p);
   FSD_LAUNCHED(c);
   FSD_CUDA(cudaGetLastError());
   const double zeta0 = 6.0 * kPi * c.eta * c.a;

@@ -576,7 +576,7 @@ void build_neighbors(Ctx &c) {
   const double4 *spos = (const double4 *)c.wpos64.p;
   for (int attempt = 0; attempt < 4; ++attempt) {
     FSD_CUDA(cudaMemsetAsync(c.cell_count.p, 0, ncells * sizeof(int), c.stream));
-    FSD_CUDA(cudaMemsetAsync(c.flags.p, 0, kFlags * sizeof(int), c.stream));
+    FSD_CUDA(cudaMemsetAsync(c.flags.p, 0, kSearchFlags * sizeof(int), c.stream));
     k_cell_count<<<ceil_div(c.Nt, 256), 256, 0, c.stream>>>(c.Nt, spos, c.L, nc, c.cell_count.p, c.cell_id.p);
     FSD_LAUNCHED(c);
     k_exclusive_scan<<<1, 1024, 0, c.stream>>>(ncells, c.cell_count.p, c.cell_start.p,
