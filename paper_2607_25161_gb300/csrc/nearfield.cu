@@ -848,8 +848,7 @@ __global__ void __launch_bounds__(256) k_contact_bead(
   const int bi = bead_body[i];
   const double reach = fmax(2.0 * a, pf.r_cut), reach2 = reach * reach;
   const float far = (float)reach2 + m2, Lf = (float)L, invL = 1.f / Lf, tf = (float)tilt;
-  // displacement to bead j: FP32 and the image (whole boxes along x, y, z);
-  // a pair within reach, which is below L/2, has the same image in FP64
+  // displacement to bead j: FP32 and the image (whole boxes along x, y, z)
   auto image = [&](int j, float *n) {
     const float4 pj = pos32[j];
     float e0 = pi.x - pj.x, e1 = pi.y - pj.y, e2 = pi.z - pj.z;
@@ -865,11 +864,19 @@ __global__ void __launch_bounds__(256) k_contact_bead(
   double f0 = 0.0, f1 = 0.0, f2 = 0.0;
   auto take = [&](int j) {
     float nf[3];
-    image(j, nf);
+    const bool edge = image(j, nf) > 0.2499f * Lf * Lf;
     const double4 q = pos[j];
-    const double ny = (double)nf[1];
-    const double d0 = fma(-(double)nf[0], L, fma(-ny, tilt, p.x - q.x));
-    const double d1 = fma(-ny, L, p.y - q.y), d2 = fma(-(double)nf[2], L, p.z - q.z);
+    double d0 = p.x - q.x, d1 = p.y - q.y, d2 = p.z - q.z;
+    if (edge) {
+      // a component may be within FP32 rounding of L/2: the image of FP64
+      le_image(d0, d1, d2, L, tilt);
+    } else {
+      // closer pairs have the same image in FP64
+      const double ny = (double)nf[1];
+      d0 = fma(-(double)nf[0], L, fma(-ny, tilt, d0));
+      d1 = fma(-ny, L, d1);
+      d2 = fma(-(double)nf[2], L, d2);
+    }
     const double r2 = d0 * d0 + d1 * d1 + d2 * d2;
     if (r2 >= reach2 || r2 == 0.0) return;
     const double r = sqrt(r2), ir = 1.0 / r;
