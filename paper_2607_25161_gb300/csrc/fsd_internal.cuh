@@ -271,6 +271,29 @@ __device__ __forceinline__ void le_image(double &d0, double &d1, double &d2, dou
   d2 -= L * rint(d2 / L);
 }
 
+// ------------------------------------------------------ inverse distance
+// 1/r and r from r^2: a reciprocal square root estimate refined by one step of
+// Halley's iteration y (1 + e/2 + 3 e^2/8), e = 1 - r^2 y^2, of cubic order:
+// the estimate's error of a few 1e-7 becomes FP64 rounding (e^3 ~ 1e-19), and
+// FP32's own estimate FP32 rounding.  In FP64 eight operations of the pipe that
+// bounds the pair sum instead of a square root and a division (about
+// twenty-five); the FP64 estimate takes any length unit (an FP32 one lost
+// every digit of r^2 below 1e-45, r of 1e-22 units).
+template <typename T>
+__device__ __forceinline__ T inv_sqrt(T r2);
+template <>
+__device__ __forceinline__ float inv_sqrt<float>(float r2) {
+  const float y = rsqrtf(r2), e = fmaf(-r2 * y, y, 1.f);
+  return fmaf(y * e, fmaf(0.375f, e, 0.5f), y);
+}
+template <>
+__device__ __forceinline__ double inv_sqrt<double>(double r2) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+  const double e = fma(-r2 * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
 // ------------------------------------------------- counter-based normals
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC 2011): ten rounds of two
 // 32x32 -> 64-bit multiplications with the Weyl key schedule; the Brownian

@@ -718,24 +718,6 @@ __device__ __forceinline__ void free_phi(const T inv, const T a2, const T c8, T 
   ph[6] = c8 * (T(-15) * i7 + T(42) * a2 * i9);
 }
 
-// 1/r and r from r^2: a reciprocal square root estimate refined by one step of
-// Halley's iteration y (1 + e/2 + 3 e^2/8), e = 1 - r^2 y^2, of cubic order: a
-// single-precision estimate reaches FP64 rounding (e^3 ~ 1e-20), and FP32's
-// own estimate FP32 rounding.  One FP64 pipe pass of eight operations instead
-// of a square root and a division (about twenty-five).
-template <typename T>
-__device__ __forceinline__ T inv_sqrt(T r2);
-template <>
-__device__ __forceinline__ float inv_sqrt<float>(float r2) {
-  const float y = rsqrtf(r2), e = fmaf(-r2 * y, y, 1.f);
-  return fmaf(y * e, fmaf(0.375f, e, 0.5f), y);
-}
-template <>
-__device__ __forceinline__ double inv_sqrt<double>(double r2) {
-  const double y = (double)rsqrtf((float)r2), e = fma(-r2 * y, y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
 // Wave-part radial functions from the Chebyshev-fitted table (monomials in
 // t in [-1, 1] per interval), all seven functions per Horner step.  The pad
 // slot of power 0 holds 2 iv + 1, so that t = 2 r / h - (2 iv + 1) is one
@@ -965,7 +947,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_realspace(
   // (self term, strain coordinates, rigid-body constraint, in FP64) are then
   // finished by eleven lanes: an FP64 instruction costs the SM the same for one
   // lane as for 32, and on one lane per group this epilogue was some 45 of them
-  // per two beads.  With the reciprocal square root above, FP32 on 32768 beads
+  // per two beads.  With inv_sqrt, FP32 on 32768 beads
   // 122 -> 115 us per application; FP64 (whose pair loop it bounds: also the
   // image test and 128 registers instead of spilling at 64) 3.07 -> 2.75 ms.
   T r6[6], r3[3];
