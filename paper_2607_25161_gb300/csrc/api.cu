@@ -663,13 +663,13 @@ static void setup_impl(Ctx &c, int64_t n_beads, const double *bead_pos, const in
 // lubrication blocks, Schur LUs (Alg. 1 step 1), and the FP32 spreading's tile
 // lists where the solve applies the FP32 operator (another FP32 application
 // builds them itself).  A mobility application takes the lists alone: the
-// lubrication kernels and, in FP64, the tiles were 0.15 ms of a 1.6 ms call.
+// lubrication kernels and the tiles were 0.15 ms of a 1.6 ms FP64 call.
 static void prepare(Ctx &c, bool lubrication = true) {
   c.last_warning = FSD_OK;
   launch_wrap_positions(c);
   build_neighbors(c);
   if (lubrication) build_lubrication(c);
-  if (c.spread_gather && !c.tiles_valid && c.prm.precision == FSD_MIXED) build_spread_tiles(c);
+  if (lubrication && c.spread_gather && !c.tiles_valid && c.prm.precision == FSD_MIXED) build_spread_tiles(c);
 }
 
 static void fill_stats(Ctx &c, fsd_stats *st, const KStats &k, double rel, double ms) {
