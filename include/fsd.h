@@ -217,7 +217,8 @@ void fsd_default_params(fsd_params *p);
  * every id in 0..N-1 used at least once.  The body frame is the bead layout
  * given here (orientation quaternion = identity), centred on the bead
  * centroid X (equal bead masses, Sec. 2.3.1).  cuda_stream: a cudaStream_t or
- * NULL for a stream the context creates.  On failure *ctx is NULL. */
+ * NULL for a stream the context creates; device arrays given here are read
+ * after the work queued on a stream given.  On failure *ctx is NULL. */
 fsd_status fsd_setup(fsd_ctx **ctx, int64_t n_beads, const double *bead_pos,
                      const int32_t *agg_id, const fsd_params *p,
                      void *cuda_stream);

@@ -417,7 +417,9 @@ static void setup_impl(Ctx &c, int64_t n_beads, const double *bead_pos, const in
       FSD_CUDA(cudaEventCreateWithFlags(&c.ev_join, cudaEventDisableTiming));
     }
   }
-  // ---- inputs to host
+  // ---- inputs to host (device arrays: after the caller's work on the stream given,
+  // which a blocking copy does not wait for by itself)
+  if (!c.own_stream) FSD_CUDA(cudaStreamSynchronize(c.stream));
   std::vector<double> pos(3 * (size_t)c.Nt);
   std::vector<int32_t> ids(c.Nt);
   if (is_device_ptr(bead_pos))
@@ -1669,6 +1671,7 @@ fsd_status fsd_setup_batch(fsd_batch **batch, int n_sys, const int64_t *bead_off
   try {
     b = new fsd_batch();
     b->user = (cudaStream_t)cuda_stream;
+    if (b->user) FSD_CUDA(cudaStreamSynchronize(b->user));  // device inputs may be in the making there
     if (const char *e = std::getenv("FSD_BATCH_THREADS")) b->host_threads = std::max(1, std::atoi(e));
     b->bead_off.assign(bead_offsets, bead_offsets + n_sys + 1);
     b->agg_off.assign(1, 0);

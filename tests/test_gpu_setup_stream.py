@@ -1,0 +1,37 @@
+"""A set-up on the caller's stream reads device positions after the work that
+the caller has queued there: positions written behind 0.2 s of other work on a
+non-blocking stream give the context that the same positions on the host give."""
+
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def test_setup_waits_for_positions_on_the_callers_stream():
+    torch = pytest.importorskip("torch")
+    import __graft_entry__ as g
+
+    g.build()
+    import paper_2607_25161_gb300 as pkg
+
+    pos, body, L = synth.suspension(30, 4, 0.1, 5)
+    F = np.random.default_rng(5).normal(size=(len(pos), 11))
+    s = pkg.Suspension(pos, body, L, xi=0.9)
+    want = s.apply_mobility(F)
+    s.close()
+    src = torch.tensor(pos, dtype=torch.float64, device="cuda")
+    dev = torch.full_like(src, 1.0)
+    ids = torch.tensor(body, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(400_000_000)
+        dev.copy_(src)
+    s = pkg.Suspension(dev, ids, L, stream=side.cuda_stream, xi=0.9)
+    got = s.apply_mobility(F)
+    s.close()
+    # FP64 spreading sums with atomics: rounding of the order of summation
+    assert np.linalg.norm(got - want) <= 1e-12 * np.linalg.norm(want)
