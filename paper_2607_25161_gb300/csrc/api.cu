@@ -417,9 +417,7 @@ static void setup_impl(Ctx &c, int64_t n_beads, const double *bead_pos, const in
       FSD_CUDA(cudaEventCreateWithFlags(&c.ev_join, cudaEventDisableTiming));
     }
   }
-  // ---- inputs to host (device arrays: after the caller's work on the stream given,
-  // which a blocking copy does not wait for by itself)
-  if (!c.own_stream) FSD_CUDA(cudaStreamSynchronize(c.stream));
+  // ---- inputs to host
   std::vector<double> pos(3 * (size_t)c.Nt);
   std::vector<int32_t> ids(c.Nt);
   if (is_device_ptr(bead_pos))
@@ -1159,6 +1157,9 @@ fsd_status fsd_setup(fsd_ctx **ctx, int64_t n_beads, const double *bead_pos, con
   *ctx = nullptr;
   fsd_ctx *cx = nullptr;
   FSD_API_TRY
+  // device inputs may be in the making on the caller's stream, which the blocking
+  // copies of the set-up (and the tuner's) do not wait for by themselves
+  if (cuda_stream) FSD_CUDA(cudaStreamSynchronize((cudaStream_t)cuda_stream));
   fsd_params q = *p;
   double tuned = 0.0;
   if ((q.flags & FSD_FLAG_AUTOTUNE) && q.xi <= 0 && q.rc <= 0 && q.grid <= 0)

@@ -10,7 +10,8 @@ import synth
 pytestmark = pytest.mark.gpu
 
 
-def test_setup_waits_for_positions_on_the_callers_stream():
+@pytest.mark.parametrize("tuned", [False, True])
+def test_setup_waits_for_positions_on_the_callers_stream(tuned):
     torch = pytest.importorskip("torch")
     import __graft_entry__ as g
 
@@ -19,8 +20,15 @@ def test_setup_waits_for_positions_on_the_callers_stream():
 
     pos, body, L = synth.suspension(30, 4, 0.1, 5)
     F = np.random.default_rng(5).normal(size=(len(pos), 11))
-    s = pkg.Suspension(pos, body, L, xi=0.9)
-    want = s.apply_mobility(F)
+    # the tuner reads the positions too; its choice of xi follows its timing, so
+    # only the lubrication operator, which no tuned parameter enters, is compared
+    prm = dict(flags=pkg.FSD_FLAG_AUTOTUNE, lub_cutoff=3.0) if tuned else dict(xi=0.9)
+
+    def look(s):
+        return s.apply_lubrication(F[:30, :6]) if tuned else s.apply_mobility(F)
+
+    s = pkg.Suspension(pos, body, L, **prm)
+    want = look(s)
     s.close()
     src = torch.tensor(pos, dtype=torch.float64, device="cuda")
     dev = torch.full_like(src, 1.0)
@@ -30,8 +38,8 @@ def test_setup_waits_for_positions_on_the_callers_stream():
     with torch.cuda.stream(side):
         torch.cuda._sleep(400_000_000)
         dev.copy_(src)
-    s = pkg.Suspension(dev, ids, L, stream=side.cuda_stream, xi=0.9)
-    got = s.apply_mobility(F)
+    s = pkg.Suspension(dev, ids, L, stream=side.cuda_stream, **prm)
+    got = look(s)
     s.close()
     # FP64 spreading sums with atomics: rounding of the order of summation
     assert np.linalg.norm(got - want) <= 1e-12 * np.linalg.norm(want)
