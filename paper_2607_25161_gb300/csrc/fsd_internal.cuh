@@ -83,10 +83,15 @@ struct OpData {
   DBuf<T> table;      // real-space radial table [nint][power][function padded to 8]
   T self_real[3];     // real-space self mobilities (translation, rotation, strain)
   DBuf<T> grid;       // spread densities, planar: [6][n^3]
-  DBuf<T> spec;       // half spectra, planar: [6][n][n][n/2 + 1] complex
-  DBuf<T> gout;       // velocity fields for interpolation, interleaved: [n^3][8] (6 used)
-  DBuf<T> green;      // [m = kx^2+ky^2+kz^2][3]: (A fM^2, A fM fD, A fD^2)
-  DBuf<T> twiddle;    // [n] complex: exp(-2 pi i t / n)
+  // (two-factor: the grid sizes of fft.cuh's kernels; staged: the others)
+  DBuf<T> spec;       // two-factor: three full complex fields [3][z][kx][y];
+                      // staged: half spectra, planar, [6][n][n][n/2 + 1] complex
+  DBuf<T> gout;       // velocity fields for interpolation: two-factor FP32 in bricks or
+                      // planar (kFftBricks), else interleaved [n^3][8] (6 used)
+  DBuf<T> green;      // by m = kx^2+ky^2+kz^2: (A fM^2, A fM fD, A fD^2); two-factor: halved,
+                      // and in FP64 four wide with 1/m (staged, and FP32: three wide)
+  DBuf<T> twiddle;    // two-factor: exp(-2 pi i j k1 / n) [k1 < R1][j < R2]; staged: a table
+                      // per stage (make_plan)
   DBuf<T> pos;        // wrapped positions [Nt][4] (x, y, z, 0)
   DBuf<T> lever;      // r_b = x_b - X_J [Nt][4]
   DBuf<T> packed;     // per bead (x, y, z, F, L, S6, 0) in the operator precision [Nt][16]
@@ -101,7 +106,7 @@ enum ProfGroup {
   PG_SPREAD,    // Gaussian spreading
   PG_FFT,       // FFT passes incl. the fused Green's function
   PG_INTERP,    // interpolation
-  PG_BODY,      // aggregate rows: constraint gather + lubrication BSR
+  PG_BODY,      // aggregate rows: constraint gather + lubrication pairs
   PG_PRECOND,   // preconditioner apply
   PG_KRYLOV,    // Arnoldi dots / updates / scaling
   PG_NEIGHBOR,  // cell and neighbour lists
@@ -202,7 +207,7 @@ struct Ctx {
   // [kSingular] singular LU
   DBuf<int> flags;
   int *h_flags = nullptr;  // pinned
-  // ---- lubrication BSR (rows = beads; diagonal separate)
+  // ---- lubrication pairs in CSR order (rows = beads)
   DBuf<int> brow, bcol;
   DBuf<double> lpair;   // per directed pair (n, r, A, B, D, within r_p) [nnz][8]
   DBuf<float> lpair32;  // the same in FP32 (n, r/2, A, B, D, 0) [nnz][8]
@@ -369,7 +374,7 @@ void launch_wavespace(Ctx &c, const double *x, double *y,
                       bool set = false);  // y += M_w x, or y = M_w x (bead rows)
 
 // nearfield.cu
-void build_lubrication(Ctx &c);  // BSR blocks (both precisions) + Schur LU
+void build_lubrication(Ctx &c);  // pair records (both precisions; FP64 6x6 blocks for Lanczos) + Schur LU
 template <typename T>
 void launch_body_rows(Ctx &c, const double *x, double *y, bool with_lub,
                       const double *add = nullptr);  // y2 = Sigma B^T x1 - RR x2; bead rows += add

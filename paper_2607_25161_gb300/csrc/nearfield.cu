@@ -1,9 +1,9 @@
-// Near-field lubrication (BSR of 6x6 bead blocks over inter-body pairs,
-// Alg. 1 step 1), the rigid-body constraint Sigma / Sigma^T (Eq. gc,
-// Eq. sigma), the block-triangular preconditioner with one 6x6 LU per
-// aggregate (Table 1; Alg. 1 step 1), the right-hand side of Eq. spm_agg,
-// the outputs (Eq. stress_comp a, d) and the rigid-body integrator
-// (Eq. EM1-EM3).
+// Near-field lubrication (records of the inter-body pairs in CSR order; their
+// 6x6 blocks for the Lanczos sampler alone; Alg. 1 step 1), the rigid-body
+// constraint Sigma / Sigma^T (Eq. gc, Eq. sigma), the block-triangular
+// preconditioner with one 6x6 LU per aggregate (Table 1; Alg. 1 step 1), the
+// right-hand side of Eq. spm_agg, the outputs (Eq. stress_comp a, d) and the
+// rigid-body integrator (Eq. EM1-EM3).
 //
 // Pair resistance (per inter-body pair i, j; n from i to j, gap h = r - 2a,
 // eps = max(h, hmin)/a, cut-off eps_c = r_lub/a - 2):

@@ -324,9 +324,6 @@ __global__ void k_cell_fill(int Nt, const int *__restrict__ cell_id, int *cursor
   cell_beads[slot] = i;
 }
 
-// Sort each cell's bead indices (one thread per cell): with the cells
-// visited in a fixed order, every neighbour row, and so every pair sum, then
-// runs in an order that does not depend on the atomic fill.
 // Sort each segment [start[c], start[c + 1]) of `items` ascending (the
 // atomically filled cell and tile lists, so that every later sum runs in a
 // fixed order).  One warp per segment: a bitonic sort in shared memory for
@@ -630,29 +627,11 @@ void build_neighbors(Ctx &c) {
 // ============================================================ pair sum
 
 template <typename T>
-struct RS;
-template <>
-struct RS<float> {
-  using V4 = float4;
-};
-template <>
-struct RS<double> {
-  using V4 = double4;
-};
-
-template <typename T>
 __device__ __forceinline__ T rint_t(T x);
 template <>
 __device__ __forceinline__ float rint_t<float>(float x) { return rintf(x); }
 template <>
 __device__ __forceinline__ double rint_t<double>(double x) { return rint(x); }
-
-template <typename T>
-__device__ __forceinline__ T sqrt_t(T x);
-template <>
-__device__ __forceinline__ float sqrt_t<float>(float x) { return sqrtf(x); }
-template <>
-__device__ __forceinline__ double sqrt_t<double>(double x) { return sqrt(x); }
 
 // Accumulate the action of one FTS pair block (given its seven radial
 // scalars) on the source moments (F, L, S) into (u, omega, e6).
@@ -1000,17 +979,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_realspace(
   }
   __syncwarp();
   }
-}
-
-template <typename T>
-static const typename RS<T>::V4 *pos_ptr(Ctx &c);
-template <>
-const double4 *pos_ptr<double>(Ctx &c) {
-  return (const double4 *)c.pos64.p;
-}
-template <>
-const float4 *pos_ptr<float>(Ctx &c) {
-  return (const float4 *)c.op32.pos.p;
 }
 
 template <typename T>

@@ -103,25 +103,24 @@ struct FftPlan {
   FftStage st[kMaxStages];
 };
 
-// Stages 16^a 9^b 8^c 4^d 2^e 3^f 5^g with big_radix (the largest register
+// Stages 16^a 9^b 8^c 4^d 2^e 3^f 5^g (the largest register
 // DFTs first: fewer passes through shared memory, and fewer twiddle products,
 // which is what an FP64 transform spends its time on where FP64 runs at 1/74
-// of the FP32 rate), else 4^d 2^e 3^f 5^g; per stage the twiddles
+// of the FP32 rate); per stage the twiddles
 // exp(-2 pi i r k / (Ns R)), r = 1..R-1, k < Ns, stored contiguously
 // (complex) from toff.
-static FftPlan make_plan(int n, std::vector<double> *tw, bool big_radix) {
+static FftPlan make_plan(int n, std::vector<double> *tw) {
   FftPlan p{};
   p.n = n;
   p.fn = make_fastdiv(n);
   p.fnh = make_fastdiv(n / 2 + 1);
   int m = n, k = 0;
   std::vector<int> radices;
-  if (big_radix)
-    for (int f : {16, 9, 8})
-      while (m % f == 0) {
-        radices.push_back(f);
-        m /= f;
-      }
+  for (int f : {16, 9, 8})
+    while (m % f == 0) {
+      radices.push_back(f);
+      m /= f;
+    }
   while (m % 4 == 0) {
     radices.push_back(4);
     m /= 4;
@@ -1658,7 +1657,7 @@ void build_wave(Ctx &c) {
         tw.push_back(std::sin(ang));
       }
   } else {
-    make_plan(n, &tw, true);
+    make_plan(n, &tw);
   }
   upload_as(c, c.op64.twiddle, tw);
   upload_as(c, c.op32.twiddle, tw);
@@ -1791,7 +1790,7 @@ static void wave_tail(Ctx &c, OpData<T> &op, Cx<T> *spec, double *y, bool set) {
       FSD_LAUNCHED(c);
       FSD_CUDA(cudaGetLastError());
     } else {
-      const FftPlan plan = make_plan(n, nullptr, true);
+      const FftPlan plan = make_plan(n, nullptr);
       const int nh = n / 2 + 1, threads = 256, ntw = plan.ntw;
       const int LTXy = fit_log2_lines<T>(sizeof(T) == 8 ? 3 : 4, 1, n, ntw);
       const int TXy = 1 << LTXy;
@@ -1975,7 +1974,7 @@ void launch_wavespace(Ctx &c, const double *x, double *y, bool set) {
     FSD_LAUNCHED(c);
     FSD_CUDA(cudaGetLastError());
   } else {
-    const FftPlan plan = make_plan(n, nullptr, true);
+    const FftPlan plan = make_plan(n, nullptr);
     const int nh = n / 2 + 1, threads = 256, ntw = plan.ntw;
     const int LTXy = fit_log2_lines<T>(sizeof(T) == 8 ? 3 : 4, 1, n, ntw);
     const int TXy = 1 << LTXy;
@@ -2039,7 +2038,7 @@ void launch_brownian_wave(Ctx &c, const double *field, uint64_t seed, uint64_t s
       }
       f->z_brown(c.stream, (Cplx<T> *)spec, (const Cplx<T> *)op.twiddle.p, b);
     } else {
-      const FftPlan plan = make_plan(n, nullptr, true);
+      const FftPlan plan = make_plan(n, nullptr);
       const int LTX = fit_log2_lines<T>(2, 6, n, plan.ntw);
       const int TX = 1 << LTX;
       const size_t sm = (size_t)(plan.ntw + 2 * 6 * TX * fft_ls(n)) * sizeof(Cx<T>);
@@ -2077,7 +2076,7 @@ template void launch_brownian_wave<double>(Ctx &, const double *, uint64_t, uint
 // process's device footprint after start-up, or real-time loops where an
 // allocation (and the implicit synchronisation cudaMalloc / cudaFree can
 // cause) is not allowed.  For them fsd_apply_wave_noalloc applies the FP32
-// wave-space operator with every intermediate (density grids, half spectra,
+// wave-space operator with every intermediate (density grids, spectra,
 // velocity grid, Green's table, twiddles, staged bead data) placed in one
 // file-scope device array of fixed size.  The array exists on every device
 // that loads this library and stays there until the process exits.  All
