@@ -1778,12 +1778,20 @@ static fsd_status batch_run(fsd_batch *b, const double *ft, const double *shear_
       } catch (const Invalid &e) {
         err[s] = e.msg;
         st[s] = FSD_EINVAL;
+      } catch (const std::exception &) {  // nothing may leave the thread
+        err[s] = "no host memory";
+        st[s] = FSD_ENOMEM;
       }
     }
   };
   const int nthreads = std::max(1, std::min({ns, b->host_threads}));
   std::vector<std::thread> pool;
-  for (int t = 1; t < nthreads; ++t) pool.emplace_back(worker);
+  try {
+    pool.reserve(nthreads);
+    for (int t = 1; t < nthreads; ++t) pool.emplace_back(worker);
+  } catch (const std::exception &) {
+    // no more threads to be had: those that run, this one at least, take the systems
+  }
   worker();
   for (auto &th : pool) th.join();
   for (int s : b->order) {
@@ -1804,6 +1812,9 @@ static fsd_status batch_run(fsd_batch *b, const double *ft, const double *shear_
     } catch (const Invalid &e) {
       err[s] = e.msg;
       st[s] = FSD_EINVAL;
+    } catch (const std::exception &) {
+      err[s] = "no host memory";
+      st[s] = FSD_ENOMEM;
     }
   }
   if (b->user)
@@ -1838,6 +1849,9 @@ fsd_status fsd_solve_batch(fsd_batch *b, const double *agg_force_torque, const d
   } catch (const CudaError &e) {
     b->last_error = std::string(e.what) + ": " + cudaGetErrorString(e.e);
     return FSD_ECUDA;
+  } catch (const std::exception &) {
+    b->last_error = "host allocation failed";
+    return FSD_ENOMEM;
   }
 }
 
@@ -1858,6 +1872,9 @@ fsd_status fsd_step_batch(fsd_batch *b, const double *agg_force_torque, const do
   } catch (const CudaError &e) {
     b->last_error = std::string(e.what) + ": " + cudaGetErrorString(e.e);
     return FSD_ECUDA;
+  } catch (const std::exception &) {
+    b->last_error = "host allocation failed";
+    return FSD_ENOMEM;
   }
 }
 
