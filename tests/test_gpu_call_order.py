@@ -50,5 +50,7 @@ def test_mobility_between_forces_and_solve_changes_nothing(pkg):
     s.apply_mobility(np.ones((160, 11)), precision=pkg.FSD_MIXED)
     got = s.solve(ft, 1.0)[:2]
     s.close()
-    for x, y in zip(got, want):  # the same kernels on the same lists: repeats exactly
-        assert np.array_equal(x, y)
+    # the same kernels on the same lists (a second refinement sweep's FP64
+    # spreading sums with atomics)
+    for x, y in zip(got, want):
+        assert np.linalg.norm(x - y) <= 1e-9 * np.linalg.norm(y)
